@@ -29,6 +29,7 @@ struct Batch {
         int K = 0;
         bool dense = false;
         bool contig = false;  // every plan of the group has a contiguous residual stream
+        ContigMode mode;      // form of the captured launch when contig
         std::vector<int> graphs;
         ExecDesc* descs_dev = nullptr;
         int32_t* queue = nullptr;
@@ -221,20 +222,40 @@ ns_status_t ns_batch_execute(ns_batch_t b, const void* const* Bs, float* const* 
             NS_CUDA_TRY(cudaStreamSynchronize(st));  // d is a local buffer
         }
     }
+    // the form of each contiguous-stream launch: 32-byte loads need every B of the group aligned
+    for (auto& G : Bt->groups) {
+        ContigMode m;
+        for (int g : G.graphs) m.b32 = m.b32 && (reinterpret_cast<uintptr_t>(Bs[g]) & 31u) == 0;
+        m.coop = G.n_items * kExecWarps <= 8 * (int64_t)num_sms(Bt->plans[G.graphs[0]]->device);
+        m.W = G.W;
+        if (Bt->exec && G.contig && m.b32 != G.mode.b32) {  // captured for the other alignment
+            NS_CUDA_TRY(cudaStreamSynchronize(Bt->graph_stream));
+            cudaGraphExecDestroy(Bt->exec);
+            cudaGraphDestroy(Bt->graph);
+            Bt->exec = nullptr;
+            Bt->graph = nullptr;
+        }
+        G.mode = m;
+    }
     if (!Bt->exec) {
         // capture every group's persistent launch once; later calls replay the graph
-        for (auto& G : Bt->groups)  // occupancy queries and attributes outside the capture
-            NS_TRY(exec_prepare(G.n_items, G.K, G.TM, G.TK, Bt->dtype == NS_BF16, Bt->hint, G.dense, &G.grid, G.W,
-                                G.contig));
+        for (auto& G : Bt->groups) {  // occupancy queries and attributes outside the capture
+            const bool bf16 = Bt->dtype == NS_BF16;
+            if (G.contig) NS_TRY(contig_prepare(G.n_items, G.K, bf16, G.mode, &G.grid));
+            else NS_TRY(exec_prepare(G.n_items, G.K, G.TM, G.TK, bf16, Bt->hint, G.dense, &G.grid, G.W));
+        }
         // the caller's stream may be the legacy default stream, which cannot be captured: record
         // the launches on a private stream once; the graph then replays on the caller's stream
         if (!Bt->cap_stream) NS_CUDA_TRY(cudaStreamCreateWithFlags(&Bt->cap_stream, cudaStreamNonBlocking));
         NS_CUDA_TRY(cudaStreamBeginCapture(Bt->cap_stream, cudaStreamCaptureModeThreadLocal));
         ns_status_t r = NS_OK;
         for (auto& G : Bt->groups) {
-            r = exec_launch(G.descs_dev, G.queue, G.queue_desc, G.n_items, G.ctrl, G.K, G.TM, G.TK,
-                            Bt->dtype == NS_BF16, Bt->hint, G.dense, &G.grid, Bt->cap_stream, nullptr, G.W,
-                            G.contig);
+            if (G.contig)
+                r = contig_launch(G.descs_dev, G.queue, G.queue_desc, G.n_items, G.ctrl, G.K, Bt->dtype == NS_BF16,
+                                  G.mode, &G.grid, Bt->cap_stream);
+            else
+                r = exec_launch(G.descs_dev, G.queue, G.queue_desc, G.n_items, G.ctrl, G.K, G.TM, G.TK,
+                                Bt->dtype == NS_BF16, Bt->hint, G.dense, &G.grid, Bt->cap_stream, nullptr, G.W);
             if (r != NS_OK) break;
         }
         cudaGraph_t graph = nullptr;

@@ -16,127 +16,11 @@
 //
 // L2 policy (Section 6.2.1 hot-B staging in GPU form): A's arrays and C are streamed with an
 // evict-first policy, B rows are loaded with evict-last so that reused B rows stay in L2.
-#include <type_traits>
-
 #include "ns_internal.cuh"
+#include "ns_mem.cuh"
 #include "ns_ptx.cuh"
 
 namespace ns {
-
-// ---------------------------------------------------------------------------------------------
-// memory helpers with L2 cache policies
-// ---------------------------------------------------------------------------------------------
-struct Policies {
-    uint64_t first, last;
-};
-
-__device__ __forceinline__ Policies make_policies()
-{
-    Policies p;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p.first));
-    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p.last));
-    return p;
-}
-
-template <bool HINT>
-__device__ __forceinline__ int32_t ld_stream_i32(const int32_t* p, uint64_t pol)
-{
-    int32_t v;
-    if (HINT)
-        asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.b32 %0, [%1], %2;"
-                     : "=r"(v) : "l"(p), "l"(pol));
-    else
-        v = __ldg(p);
-    return v;
-}
-
-template <bool HINT>
-__device__ __forceinline__ float ld_stream_f32(const float* p, uint64_t pol)
-{
-    float v;
-    if (HINT)
-        asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.f32 %0, [%1], %2;"
-                     : "=f"(v) : "l"(p), "l"(pol));
-    else
-        v = __ldg(p);
-    return v;
-}
-
-// Four consecutive B elements as loaded: 16 B of FP32 or 8 B of BF16.  Rings of gathers keep
-// this raw form and widen a vector only where it is used: a conversion next to its load would
-// wait for the load there and leave one gather in flight instead of the ring's depth.
-template <bool BF16>
-using BRaw = std::conditional_t<BF16, uint2, float4>;
-
-template <bool BF16, bool HINT>
-__device__ __forceinline__ BRaw<BF16> ld_braw(const void* p, uint64_t pol)
-{
-    BRaw<BF16> r;
-    if constexpr (!BF16) {
-        if (HINT)
-            asm volatile("ld.global.nc.L2::cache_hint.v4.f32 {%0,%1,%2,%3}, [%4], %5;"
-                         : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w) : "l"(p), "l"(pol));
-        else
-            r = __ldg(reinterpret_cast<const float4*>(p));
-    } else {
-        if (HINT)
-            asm volatile("ld.global.nc.L2::cache_hint.v2.b32 {%0,%1}, [%2], %3;"
-                         : "=r"(r.x), "=r"(r.y) : "l"(p), "l"(pol));
-        else
-            r = __ldg(reinterpret_cast<const uint2*>(p));
-    }
-    return r;
-}
-
-// 16 raw bytes (eight BF16 columns)
-template <bool HINT>
-__device__ __forceinline__ uint4 ld_b16(const void* p, uint64_t pol)
-{
-    uint4 r;
-    if (HINT)
-        asm volatile("ld.global.nc.L2::cache_hint.v4.b32 {%0,%1,%2,%3}, [%4], %5;"
-                     : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p), "l"(pol));
-    else
-        r = __ldg(reinterpret_cast<const uint4*>(p));
-    return r;
-}
-
-template <bool BF16>
-__device__ __forceinline__ BRaw<BF16> braw_zero()
-{
-    if constexpr (BF16) return make_uint2(0u, 0u);
-    else return make_float4(0.f, 0.f, 0.f, 0.f);
-}
-
-__device__ __forceinline__ float4 widen(const float4& v) { return v; }
-__device__ __forceinline__ float4 widen(const uint2& v)  // BF16 is the high half of an FP32
-{
-    return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u),
-                       __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
-}
-
-template <bool HINT>
-__device__ __forceinline__ void st_c4(float* p, float4 v, uint64_t pol)
-{
-    if (HINT)
-        asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1,%2,%3,%4}, %5;"
-                     :: "l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "l"(pol) : "memory");
-    else
-        *reinterpret_cast<float4*>(p) = v;
-}
-
-__device__ __forceinline__ float4 f4_fma(float a, float4 b, float4 c)
-{
-    c.x = fmaf(a, b.x, c.x);
-    c.y = fmaf(a, b.y, c.y);
-    c.z = fmaf(a, b.z, c.z);
-    c.w = fmaf(a, b.w, c.w);
-    return c;
-}
-__device__ __forceinline__ float4 f4_add(float4 a, float4 b)
-{
-    return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
-}
 
 // ---------------------------------------------------------------------------------------------
 // delivering one piece of an output row
@@ -265,8 +149,7 @@ __device__ __forceinline__ void group_reduce(float4 (&acc)[VPL])
 }
 
 // split-row delivery out of line (rare): keeps the inlined row flush of the stream path small
-// PAIR: the lane holds vectors 2 lane and 2 lane + 1 (adjacent), otherwise lane and lane + 32
-template <int VPL, bool HINT, bool PAIR = false>
+template <int VPL, bool HINT>
 __device__ __noinline__ void deliver_split_row(const ExecDesc& D, int32_t row, int32_t s, int32_t c,
                                                float4 a0, float4 a1, int lane, uint64_t pol_first)
 {
@@ -274,7 +157,7 @@ __device__ __noinline__ void deliver_split_row(const ExecDesc& D, int32_t row, i
     const int32_t np = __ldg(D.split_np + s);
     const int32_t piece = c - __ldg(D.split_base + s);
     float* slot0 = D.slots + (int64_t)__ldg(D.split_slot + s) * D.K;
-    const int v0 = PAIR ? 2 * lane : lane, v1 = PAIR ? 2 * lane + 1 : lane + 32;
+    const int v0 = lane, v1 = lane + 32;
     if (v0 < nv) __stcg(reinterpret_cast<float4*>(slot0 + (int64_t)piece * D.K + 4 * v0), a0);
     if (VPL > 1 && v1 < nv) __stcg(reinterpret_cast<float4*>(slot0 + (int64_t)piece * D.K + 4 * v1), a1);
     __threadfence();
@@ -287,7 +170,7 @@ __device__ __noinline__ void deliver_split_row(const ExecDesc& D, int32_t row, i
     float* crow = D.C + (int64_t)row * D.ldc;
 #pragma unroll
     for (int q = 0; q < VPL; ++q) {
-        const int v = PAIR ? 2 * lane + q : lane + 32 * q;
+        const int v = lane + 32 * q;
         if (v < nv) {
             float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
             for (int p = 0; p < np; ++p)
@@ -520,18 +403,13 @@ __device__ void residual_chunk_staged(const ExecDesc& D, int32_t c, int lane, un
             cc[u] = 0;
             vv[u] = 0.f;
             if (P < total) {
-                int64_t z;
-                if (D.rl_all) {
-                    z = rzoff[0] + P;  // one contiguous residual range
-                } else {             // the row holding P: largest r with rbeg[r] <= P
-                    int lo = 0, hi = nr;
-                    while (hi - lo > 1) {
-                        const int mid = (lo + hi) >> 1;
-                        if (rbeg[mid] <= P) lo = mid;
-                        else hi = mid;
-                    }
-                    z = rzoff[lo] + (P - rbeg[lo]);
+                int lo = 0, hi = nr;  // the row holding P: largest r with rbeg[r] <= P
+                while (hi - lo > 1) {
+                    const int mid = (lo + hi) >> 1;
+                    if (rbeg[mid] <= P) lo = mid;
+                    else hi = mid;
                 }
+                const int64_t z = rzoff[lo] + (P - rbeg[lo]);
                 if (z >= 0 && z < D.n_res) {
                     cc[u] = ld_stream_i32<HINT>(D.res_col + z, pol.first);
                     vv[u] = ld_stream_f32<HINT>(D.res_val + z, pol.first);
@@ -730,311 +608,6 @@ __global__ void __launch_bounds__(kExecThreads, DENSE ? 1 : 4) k_exec(const Exec
 }
 
 // ---------------------------------------------------------------------------------------------
-// residual-only plans whose list is every row in order (tau_tile = inf): a chunk's nonzeros are
-// one contiguous range of A and its rows are k0 .. kL themselves.  The lanes read column ids and
-// values 32 at a time, two batches ahead, into a 4-batch ring of (col, value) pairs in this warp's
-// shared memory (1 KB), which every step reads with one broadcast load; row ends and split ids
-// come 32 rows at a time; B rows are gathered through a 4-deep register ring.  At 64 registers
-// 8 CTAs (32 warps) fit on an SM: the gathers of many independent warps hide the latency spread
-// of a power-law column stream better than deeper rings in fewer warps.
-// ---------------------------------------------------------------------------------------------
-constexpr int kCRing = 4;
-
-// EPS: nonzeros per warp step (Section 7 "vector tiles merging"): the warp splits into EPS lane
-// groups of G = 32 / EPS lanes, group g takes entry P + g of the step, and a row's partial sums
-// are added across the groups when the row ends (K <= 4 G, so VPL = 1 when EPS > 1).
-// FULL: every lane of a group holds VPL whole vectors (K == 4 G VPL), so no per-lane width test.
-// HOT: the planner's hot-row map picks each gather's L2 policy; the map is read when a batch is
-// fetched and its bit travels as bit 31 of the column id.
-template <int VPL, int EPS, bool BF16, bool HINT, bool FULL, bool HOT, bool ASYNC>
-__device__ __forceinline__ void contig_chunk(const ExecDesc& D, int32_t c, int lane, const Policies& pol,
-                                             float4* park, int2* bat, float4* aring)
-{
-    // ASYNC (FP32, one 4-column vector per lane, one nonzero per step): the gathered rows land in
-    // an 8-deep ring in shared memory through cp.async (each lane copies and later reads its own
-    // 16 bytes, so no warp barrier), which doubles the rows in flight without spending registers;
-    // otherwise a kCRing-deep register ring.
-    constexpr int kR = ASYNC ? 8 : kCRing;  // ring depth (steps in flight)
-    // PAIR (BF16, K <= 128): each lane gathers 8 adjacent columns (16 bytes, vectors 2 li and
-    // 2 li + 1), so 16 lanes cover a row and the warp takes two nonzeros per step
-    constexpr bool PAIR = BF16 && VPL == 2 && EPS == 2;
-    static_assert(EPS == 1 || VPL == 1 || PAIR, "several nonzeros per step only for K <= 128");
-    constexpr int G = 32 / EPS;
-    const int g = lane / G, li = lane % G;
-    const int4 h0 = __ldg(reinterpret_cast<const int4*>(D.chunk_rec + c));
-    const int4 h1 = __ldg(reinterpret_cast<const int4*>(D.chunk_rec + c) + 1);
-    const int32_t b0 = h0.x, k0 = h0.z, kL = h0.w, z0 = h1.x, total = h1.y;
-    const int nr = kL - k0 + 1;
-    if (k0 < 0 || kL >= D.n_rl || kL < k0 || h0.y <= b0 || total < 0 || z0 < 0 ||
-        (int64_t)z0 + total > D.n_res) {
-        if (lane == 0) atomicOr(D.status, kStatusInternal);  // guard: corrupt plan
-        return;
-    }
-    const int nv = D.K >> 2;
-    constexpr int VB = BF16 ? 8 : 16;  // bytes of one 4-column vector
-    const unsigned char* const Bl = reinterpret_cast<const unsigned char*>(D.B) + (PAIR ? 2 : 1) * VB * li;
-    auto vidx = [&](int q) { return PAIR ? 2 * li + q : li + 32 * q; };  // vector q of this lane
-    const uint32_t ldb_bytes = (uint32_t)(D.ldb * (BF16 ? 2 : 4));
-
-    // ---- batches of 32 (col, value) pairs; past the end: the last column again with value 0 ----
-    const int32_t clast = total > 0 ? ld_stream_i32<HINT>(D.res_col + z0 + total - 1, pol.first) : 0;
-    auto fetch = [&](int P0, int32_t& cc, float& vv) {
-        const int P = P0 + lane;
-        cc = clast;
-        vv = 0.f;
-        if (P < total) {
-            cc = ld_stream_i32<HINT>(D.res_col + z0 + P, pol.first);
-            vv = ld_stream_f32<HINT>(D.res_val + z0 + P, pol.first);
-        }
-        if ((unsigned)cc >= (unsigned)D.n) {  // guard: never gather outside B
-            atomicOr(D.status, kStatusInternal);
-            cc = 0;
-            vv = 0.f;
-        }
-        if (HOT) cc |= (int32_t)(((__ldg(D.hot + (cc >> 5)) >> (cc & 31)) & 1u) << 31);
-    };
-    auto put = [&](int P0, int32_t cc, float vv) { bat[(P0 & 127) + lane] = make_int2(cc, __float_as_int(vv)); };
-    int32_t cr;
-    float vr;
-    fetch(0, cr, vr);
-    put(0, cr, vr);
-    fetch(32, cr, vr);
-    put(32, cr, vr);
-    fetch(64, cr, vr);  // stored when batch 32 starts
-
-    // lane j: stream end of row k0 + base + j (merge position of its end item, less b0 and the
-    // end items of the rows before it) and its split id
-    int32_t wend = 0x7fffffff, wsplit = -1;
-    auto rows = [&](int base) {
-        const int32_t k = k0 + base + lane;
-        wend = 0x7fffffff;
-        wsplit = -1;
-        if (k <= kL) {
-            wend = __ldg(D.rl_start + k + 1) - 1 - b0 - (k - k0);
-            wsplit = __ldg(D.row_split + k);
-        }
-    };
-    rows(0);
-    __syncwarp();
-
-    float4 acc[VPL];
-#pragma unroll
-    for (int q = 0; q < VPL; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-    using Raw = std::conditional_t<PAIR, uint4, BRaw<BF16>>;
-    Raw b[ASYNC ? 1 : kR][PAIR ? 1 : VPL];
-    float w[kR];
-    auto gather = [&](int2 e, int u) {
-        const uint32_t col = HOT ? ((uint32_t)e.x & 0x7fffffffu) : (uint32_t)e.x;
-        const unsigned char* row = Bl + (size_t)col * ldb_bytes;
-        const uint64_t pl = HOT ? (e.x < 0 ? pol.last : pol.first) : pol.last;
-        if constexpr (ASYNC) {
-            cp_async16<HINT>(aring + u * 32 + lane, row, FULL || li < nv, pl);
-            cp_async_commit();
-        } else if constexpr (PAIR) {  // K a multiple of 8: both vectors valid or neither
-            if (FULL || 2 * li < nv) b[u][0] = ld_b16<HINT>(row, pl);
-            else b[u][0] = make_uint4(0u, 0u, 0u, 0u);
-        } else {
-#pragma unroll
-            for (int q = 0; q < VPL; ++q) {
-                if (FULL || li + 32 * q < nv) b[u][q] = ld_braw<BF16, HINT>(row + 32 * VB * q, pl);
-                else b[u][q] = braw_zero<BF16>();
-            }
-        }
-        w[u] = __int_as_float(e.y);
-    };
-    auto bvec = [&](int u, int q) -> float4 {
-        if constexpr (ASYNC) return aring[u * 32 + lane];
-        else if constexpr (PAIR) {
-            const uint4 v = b[u][0];
-            return q == 0 ? widen(make_uint2(v.x, v.y)) : widen(make_uint2(v.z, v.w));
-        } else return widen(b[u][q]);
-    };
-    // step u of a group covers entries P + u EPS + g; the ring's first kR steps
-#pragma unroll
-    for (int u = 0; u < kR; ++u) gather(bat[u * EPS + g], u);
-
-    // Row ends inside the stream.  Only the chunk's first and last rows can be split (a middle
-    // row lies inside the chunk's merge range, so no other chunk touches it); the last one ends
-    // after the loop.  A split first row parks its partial sum in shared memory and is delivered
-    // after the loop, so the loop has no call in it and the ring keeps its registers.
-    int r = 0;
-    bool parked = false;
-    int next_end = __shfl_sync(0xffffffffu, wend, 0);
-    auto reduce_groups = [&]() {  // every group ends up with the row's full sum
-#pragma unroll
-        for (int o = G; o < 32; o <<= 1)
-#pragma unroll
-            for (int q = 0; q < VPL; ++q) {
-                acc[q].x += __shfl_xor_sync(0xffffffffu, acc[q].x, o);
-                acc[q].y += __shfl_xor_sync(0xffffffffu, acc[q].y, o);
-                acc[q].z += __shfl_xor_sync(0xffffffffu, acc[q].z, o);
-                acc[q].w += __shfl_xor_sync(0xffffffffu, acc[q].w, o);
-            }
-    };
-    auto store_row = [&]() {  // group 0 stores
-        float* crow = D.C + (int64_t)(k0 + r) * D.ldc;
-#pragma unroll
-        for (int q = 0; q < VPL; ++q) {
-            const int v = vidx(q);
-            if (g == 0 && (FULL || v < nv)) st_c4<HINT>(crow + 4 * v, acc[q], pol.first);
-        }
-    };
-    auto advance = [&]() {
-#pragma unroll
-        for (int q = 0; q < VPL; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-        ++r;
-        if ((r & 31) == 0) rows(r);
-        next_end = __shfl_sync(0xffffffffu, wend, r & 31);
-    };
-    auto flush = [&]() {  // inside the loop
-        const int32_t sp = __shfl_sync(0xffffffffu, wsplit, r & 31);
-        if (EPS > 1) reduce_groups();
-        if (sp < 0) {
-            store_row();
-        } else if (r == 0) {
-#pragma unroll
-            for (int q = 0; q < VPL; ++q) park[32 * q + lane] = acc[q];
-            parked = true;
-        } else if (lane == 0) {
-            atomicOr(D.status, kStatusInternal);  // guard: a middle row marked split
-        }
-        advance();
-    };
-    // One step: entries P .. P + EPS - 1 (ring slot u) accumulated, then the slot gathers the
-    // entries kCRing steps ahead.  A row that ends inside the step takes the groups before its end;
-    // rows ending at or after the chunk's last nonzero are left to the end.  TAIL: the step may
-    // reach past the last nonzero (those groups add nothing).
-    auto step = [&](int P, int u, const int2* e1, auto tail) {
-        constexpr bool TAIL = decltype(tail)::value;
-        const int mine = P + g;
-        if constexpr (ASYNC) cp_async_wait<kR - 1>();  // this step's row has landed
-        if (next_end >= P + EPS || next_end >= total) {
-            if (!TAIL || mine < total) {
-#pragma unroll
-                for (int q = 0; q < VPL; ++q) acc[q] = f4_fma(w[u], bvec(u, q), acc[q]);
-            }
-        } else {
-            int from = P;
-            while (next_end < P + EPS && next_end < total) {
-                if (mine >= from && mine < next_end) {
-#pragma unroll
-                    for (int q = 0; q < VPL; ++q) acc[q] = f4_fma(w[u], bvec(u, q), acc[q]);
-                }
-                if (next_end > from) from = next_end;
-                flush();
-            }
-            if (mine >= from && (!TAIL || mine < total)) {
-#pragma unroll
-                for (int q = 0; q < VPL; ++q) acc[q] = f4_fma(w[u], bvec(u, q), acc[q]);
-            }
-        }
-        gather(e1[u * EPS + g], u);
-    };
-
-    constexpr int GS = kR * EPS;  // entries per group of steps (divides the batch of 32)
-    int P = 0;
-    for (; P + GS <= total; P += GS) {
-        if ((P & 31) == 0 && P > 0) {  // batch P + 32 into the ring, batch P + 64 requested
-            put(P + 32, cr, vr);
-            __syncwarp();
-            fetch(P + 64, cr, vr);
-        }
-        const int2* e1 = bat + ((P + GS) & 127);  // entries P + GS .. P + 2 GS - 1 (GS divides 128)
-#pragma unroll
-        for (int u = 0; u < kR; ++u) step(P + u * EPS, u, e1, std::false_type{});
-    }
-    if (P < total) {  // the last partial group (its entries are already in the ring)
-        if ((P & 31) == 0 && P > 0) {
-            put(P + 32, cr, vr);
-            __syncwarp();
-        }
-        const int2* e1 = bat + ((P + GS) & 127);
-#pragma unroll
-        for (int u = 0; u < kR; ++u)
-            if (P + u * EPS < total) step(P + u * EPS, u, e1, std::true_type{});
-    }
-    if (parked) {
-        float4 p[VPL];
-#pragma unroll
-        for (int q = 0; q < VPL; ++q) p[q] = park[32 * q + lane];
-        deliver_split_row<VPL, HINT, PAIR>(D, k0, __ldg(D.row_split + k0), c, p[0], p[VPL > 1 ? VPL - 1 : 0],
-                                           lane, pol.first);
-    }
-    while (r < nr) {  // rows ending at or after the last nonzero (and the last row)
-        const int32_t sp = __shfl_sync(0xffffffffu, wsplit, r & 31);
-        if (EPS > 1) reduce_groups();
-        if (sp < 0) store_row();
-        else deliver_split_row<VPL, HINT, PAIR>(D, k0 + r, sp, c, acc[0], acc[VPL > 1 ? VPL - 1 : 0], lane,
-                                                pol.first);
-        advance();
-    }
-    if constexpr (ASYNC) cp_async_wait<0>();  // the look-ahead copies land before the ring is reused
-    __syncwarp();  // the batch ring is reused by this warp's next chunk
-}
-
-// SMEM_RING: the FP32 one-vector form may stage its gathers in the shared-memory cp.async ring
-// (pays off when the gathered rows come from DRAM; when B sits in L2 the register ring is faster).
-// HOTMAP: that ring form is built twice, with and without the planner's hot-row map, so the common
-// build carries no registers for the map (the map is a cache hint only: a build without it ignores
-// it and computes the same C); the register-ring forms read the map whenever a plan has one.
-template <int VPL, int EPS, bool BF16, bool HINT, bool SMEM_RING = true, bool HOTMAP = false>
-__global__ void __launch_bounds__(kExecThreads, VPL == 1 ? 8 : (EPS == 2 ? 6 : 5)) k_exec_contig(
-    const ExecDesc* __restrict__ descs, const int32_t* __restrict__ queue,
-    const int32_t* __restrict__ queue_desc, int64_t n_items, int32_t* ctrl,
-    const __grid_constant__ ExecDesc d0)
-{
-    constexpr bool ASYNC = SMEM_RING && VPL == 1 && EPS == 1 && !BF16;
-    constexpr bool READ_HOT = HINT && (!ASYNC || HOTMAP);
-    __shared__ float4 s_park[kExecWarps * 32 * VPL];  // one parked partial row per warp
-    __shared__ float4 s_aring[ASYNC ? kExecWarps * 8 * 32 : 1];
-    __shared__ int2 s_bat[kExecWarps * 128];          // per warp: 4 batches of 32 (col, value)
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float4* const park = s_park + warp * 32 * VPL;
-    int2* const bat = s_bat + warp * 128;
-    Policies pol{0, 0};
-    if (HINT) pol = make_policies();
-    unsigned long long* const clk = descs ? nullptr : d0.class_clock;  // single-plan launches only
-    if (clk && threadIdx.x == 0) atomicMin(clk, global_ns());
-    for (;;) {
-        int64_t u = 0;
-        if (lane == 0) u = atomicAdd(ctrl + 3, 1);
-        u = __shfl_sync(0xffffffffu, u, 0);
-        const int64_t t = u / kExecWarps;
-        if (t >= n_items) break;
-        const int32_t it = __ldg(queue + t);
-        const ExecDesc& D = descs ? descs[queue_desc ? __ldg(queue_desc + t) : 0] : d0;
-        if (it < D.n_dwin) continue;
-        const int64_t c = (int64_t)(it - D.n_dwin) * kExecWarps + (u % kExecWarps);
-        if (c >= D.n_chunks) continue;
-        if (!D.rl_all) {  // guard: launched for a plan without a contiguous residual stream
-            if (lane == 0) atomicOr(D.status, kStatusInternal);
-            continue;
-        }
-        const bool full = D.K == 128 / EPS * VPL;
-        float4* const aring = s_aring + (ASYNC ? (threadIdx.x >> 5) * 8 * 32 : 0);
-        if (READ_HOT && D.hot) {
-            if (full) contig_chunk<VPL, EPS, BF16, HINT, true, HINT, ASYNC>(D, (int32_t)c, lane, pol, park, bat, aring);
-            else contig_chunk<VPL, EPS, BF16, HINT, false, HINT, ASYNC>(D, (int32_t)c, lane, pol, park, bat, aring);
-        } else {
-            if (full) contig_chunk<VPL, EPS, BF16, HINT, true, false, ASYNC>(D, (int32_t)c, lane, pol, park, bat, aring);
-            else contig_chunk<VPL, EPS, BF16, HINT, false, false, ASYNC>(D, (int32_t)c, lane, pol, park, bat, aring);
-        }
-        if (clk && lane == 0) atomicMax(clk + 2, global_ns());
-    }
-    // the last CTA out resets the tickets for the next launch (stream order makes it visible)
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        int done = atomicAdd(ctrl + 1, 1);
-        if (done == (int)gridDim.x - 1) {
-            atomicExch(ctrl + 0, 0);
-            atomicExch(ctrl + 3, 0);
-            atomicExch(ctrl + 1, 0);
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------------------------
 // the residual list is every row in order and A itself is the residual (no window pass ran):
@@ -1043,6 +616,12 @@ bool plan_contig(const Plan* P)
 {
     return P->tune.tau_tile == kTauInf && P->st.n_dwin == 0 && P->st.n_rl == P->st.m;
 }
+
+// At most 8 chunks per SM, while the launch has 20 to 28 warps there: with one chunk a warp most
+// warps would have none, and sharing a chunk among four shortens its chain of steps (4096 rows of
+// 16, 272 chunks: 25.5 -> 13.5 us a call).  A plan's own property (not a launch's), so that a
+// request sums its rows in the same order whatever shares its launch.
+bool plan_coop(const Plan* P) { return P->st.n_chunks <= 8 * (int64_t)num_sms(P->device); }
 
 void fill_desc(const Plan* P, const void* B, int64_t ldb, float* C, int64_t ldc, ExecDesc* d)
 {
@@ -1109,53 +688,14 @@ static ExecKernel pick_kernel(int K)
     return k_exec<32, 8, BF16, HINT, DENSE>;
 }
 
-// nonzeros per warp step: as many lane groups as the K/4 vectors of a row leave room for
-template <bool BF16, bool HINT>
-static ExecKernel pick_contig(int K, bool b_in_l2, bool hot)
+static ExecKernel select_kernel(int K, bool bf16, bool hint, bool dense)
 {
-    if (K <= 32) return k_exec_contig<1, 4, BF16, HINT>;
-    if (K <= 64) return k_exec_contig<1, 2, BF16, HINT>;
-    if constexpr (BF16) {
-        if (K <= 128) return k_exec_contig<2, 2, BF16, HINT>;  // 8 columns a lane, 2 nonzeros a step
-    } else {
-        if (K <= 128 && b_in_l2) return k_exec_contig<1, 1, BF16, HINT, false>;
-    }
-    if (K <= 128) {
-        if constexpr (!BF16 && HINT)
-            if (hot) return k_exec_contig<1, 1, BF16, HINT, true, true>;
-        return k_exec_contig<1, 1, BF16, HINT>;
-    }
-    return k_exec_contig<2, 1, BF16, HINT>;
-}
-
-// contig: 0, or a residual-only launch whose plans all have a contiguous residual stream
-// (K <= 256): kContig, kContigBInL2 when B fits comfortably in L2, or kContigHot for a single
-// plan with a hot-row map
-static ExecKernel select_kernel(int K, bool bf16, bool hint, bool dense, int contig)
-{
-    if (contig && !dense && K <= 256) {
-        const bool in_l2 = contig == kContigBInL2, hot = contig == kContigHot;
-        if (bf16) return hint ? pick_contig<true, true>(K, in_l2, hot) : pick_contig<true, false>(K, in_l2, hot);
-        return hint ? pick_contig<false, true>(K, in_l2, hot) : pick_contig<false, false>(K, in_l2, hot);
-    }
     if (bf16) {
         if (hint) return dense ? pick_kernel<true, true, true>(K) : pick_kernel<true, true, false>(K);
         return dense ? pick_kernel<true, false, true>(K) : pick_kernel<true, false, false>(K);
     }
     if (hint) return dense ? pick_kernel<false, true, true>(K) : pick_kernel<false, true, false>(K);
     return dense ? pick_kernel<false, false, true>(K) : pick_kernel<false, false, false>(K);
-}
-
-int64_t l2_bytes(int device)
-{
-    static int cached[64] = {0};
-    if (device < 0 || device >= 64) return 0;
-    if (!cached[device]) {
-        int v = 0;
-        if (cudaDeviceGetAttribute(&v, cudaDevAttrL2CacheSize, device) != cudaSuccess || v <= 0) v = 1;
-        cached[device] = v;
-    }
-    return cached[device];
 }
 
 int num_sms(int device)
@@ -1172,9 +712,8 @@ int num_sms(int device)
 
 // dynamic shared memory of one execute CTA: the dense item's tiles (phase 1) or the residual
 // warps' staging rings (phase 2), whichever is larger
-static size_t exec_smem_bytes(int K, int TM, int TK, bool bf16, bool dense, int W, int contig)
+static size_t exec_smem_bytes(int K, int TM, int TK, bool bf16, bool dense, int W)
 {
-    if (contig && !dense && K <= 256) return 0;  // the contiguous-stream kernel keeps no staging
     // (L, VPL) exactly as pick_kernel chooses the instantiation
     const int nv = K / 4;
     const int L = nv <= 2 ? 2 : (nv <= 4 ? 4 : (nv <= 8 ? 8 : (nv <= 16 ? 16 : 32)));
@@ -1192,10 +731,10 @@ static size_t exec_smem_bytes(int K, int TM, int TK, bool bf16, bool dense, int 
 // Kernel attributes and the persistent grid (resident CTAs on every SM, at most n_items).
 // Must run outside stream capture.
 ns_status_t exec_prepare(int64_t n_items, int K, int TM, int TK, bool bf16, bool hint, bool dense,
-                         int* grid_out, int W, int contig)
+                         int* grid_out, int W)
 {
-    ExecKernel kern = select_kernel(K, bf16, hint, dense, contig);
-    const size_t smem = exec_smem_bytes(K, TM, TK, bf16, dense, W, contig);
+    ExecKernel kern = select_kernel(K, bf16, hint, dense);
+    const size_t smem = exec_smem_bytes(K, TM, TK, bf16, dense, W);
     if (smem > 48 * 1024) NS_TRY(dense_prepare(reinterpret_cast<const void*>(kern), smem));
     int per_sm = 0;
     NS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kExecThreads, smem));
@@ -1229,13 +768,12 @@ ns_status_t exec_prepare(int64_t n_items, int K, int TM, int TK, bool bf16, bool
 // the occupancy-derived grid between launches (0 = compute).
 ns_status_t exec_launch(const ExecDesc* descs, const int32_t* queue, const int32_t* queue_desc,
                         int64_t n_items, int32_t* ctrl, int K, int TM, int TK, bool bf16, bool hint,
-                        bool dense, int* grid_cache, cudaStream_t s, const ExecDesc* d0, int W,
-                        int contig)
+                        bool dense, int* grid_cache, cudaStream_t s, const ExecDesc* d0, int W)
 {
-    ExecKernel kern = select_kernel(K, bf16, hint, dense, contig);
-    const size_t smem = exec_smem_bytes(K, TM, TK, bf16, dense, W, contig);
+    ExecKernel kern = select_kernel(K, bf16, hint, dense);
+    const size_t smem = exec_smem_bytes(K, TM, TK, bf16, dense, W);
     int grid = grid_cache ? *grid_cache : 0;
-    if (grid == 0) NS_TRY(exec_prepare(n_items, K, TM, TK, bf16, hint, dense, &grid, W, contig));
+    if (grid == 0) NS_TRY(exec_prepare(n_items, K, TM, TK, bf16, hint, dense, &grid, W));
     if (grid_cache) *grid_cache = grid;
     if (n_items == 0) return NS_OK;
     ExecDesc dv{};
@@ -1254,15 +792,19 @@ ns_status_t exec_launch_plan(Plan* P, cudaStream_t s)
         P->exec_grid_slice = 0;
         P->exec_grid_slice_K = K;
     }
-    int contig = 0;
     if (plan_contig(P)) {
-        // B (this slice of it) within half of L2: the gathers hit L2, keep them in registers
-        const int64_t b_bytes = P->st.n * (int64_t)K * (P->dtype == NS_BF16 ? 2 : 4);
-        contig = 2 * b_bytes <= l2_bytes(P->device) ? kContigBInL2 : (P->hot_bits ? kContigHot : kContig);
+        ContigMode m;
+        m.b32 = ((reinterpret_cast<uintptr_t>(P->desc_host.B) | (uintptr_t)(P->desc_host.ldb * 4)) & 31u) == 0;
+        m.hot = P->hot_bits != nullptr;
+        m.coop = plan_coop(P);
+        m.W = P->tune.chunk_nnz;
+        // (the cached grid is the 32-byte form's; the other form is rare and asks each time)
+        return contig_launch(nullptr, P->queue, nullptr, P->st.n_items, P->ctrl, K, P->dtype == NS_BF16, m,
+                             m.b32 ? gc : nullptr, s, &P->desc_host);
     }
     return exec_launch(nullptr, P->queue, nullptr, P->st.n_items, P->ctrl, K, P->tune.TM,
                        P->tune.TK, P->dtype == NS_BF16, P->tune.l2_hints != 0, P->st.n_dwin > 0,
-                       gc, s, &P->desc_host, P->tune.chunk_nnz, contig);
+                       gc, s, &P->desc_host, P->tune.chunk_nnz);
 }
 
 }  // namespace ns

@@ -102,9 +102,11 @@ struct Arena {
 // part of the canonical plan): merge range [b0, b1), residual-list rows k0 .. kL with an item in
 // the range, the residual index of the chunk's first nonzero (the whole chunk's nonzeros are
 // z0 .. z0 + total - 1 when the residual list is every row in order) and its nonzero count.
+// `flags`: kChunkHeadCut when row k0 starts before b0, kChunkTailCut when row kL ends after b1.
 struct alignas(32) ChunkRec {
-    int32_t b0, b1, k0, kL, z0, total, pad0, pad1;
+    int32_t b0, b1, k0, kL, z0, total, flags, pad;
 };
+constexpr int32_t kChunkHeadCut = 1, kChunkTailCut = 2;
 
 struct ExecDesc {
     // residual CSR and its chunks
@@ -134,7 +136,7 @@ struct ExecDesc {
     const int32_t* split_slot;
     const int32_t* split_base;
     float* slots;        // n_slots * K floats
-    int32_t* split_cnt;  // n_split arrival counters (zero between launches)
+    int32_t* split_cnt;  // n_split * contig_slices(K) arrival counters (zero between launches)
     // operands
     const void* B;
     float* C;
@@ -199,7 +201,7 @@ struct Plan {
     // execution scratch
     float* slots = nullptr;
     int32_t* split_cnt = nullptr;
-    int32_t* ctrl = nullptr;       // [0] ticket, [1] CTAs done, [2] status, [3..] scalars
+    int32_t* ctrl = nullptr;       // [0] ticket, [1] CTAs done, [2] status, [3] chunk ticket, [4..5] 64-bit chunk ticket
     unsigned long long* class_clock = nullptr;  // set while the rebalance loop times the launch
     ExecDesc desc_host{};           // the single-plan descriptor (a kernel parameter)
     bool desc_valid = false;
@@ -226,12 +228,17 @@ ns_status_t window_pass(Plan* P, WindowResult* W, cudaStream_t s);
 __host__ __device__ inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 int num_sms(int device);
-int64_t l2_bytes(int device);
 
-// residual-only launch modes of exec_launch / exec_prepare (`contig`)
-constexpr int kContig = 1;       // contiguous residual stream
-constexpr int kContigBInL2 = 2;  // the same, with B small enough to stay in L2
-constexpr int kContigHot = 3;    // kContig, single plan with a hot-row map (l2_hints = 2)
+// form of a contiguous-stream launch (ns_contig.cu)
+struct ContigMode {
+    bool b32 = true;    // every row of B starts on a 32-byte boundary
+    bool hot = false;   // single plan with a hot-row map (l2_hints = 2)
+    bool coop = false;  // the warps of a CTA share a chunk (plan_coop)
+    int W = 256;        // chunk_nnz of the launch's plans
+};
+// Column slices of a contiguous-stream launch: one pass up to K = 256, then 128 columns a slice,
+// so that a slice's rows of B stay in L2 and no lane group is wider than a warp.
+__host__ __device__ inline int contig_slices(int K) { return K <= 256 ? 1 : (K + 127) / 128; }
 
 // planner entry (ns_plan.cu)
 ns_status_t plan_build(Plan* P, const ns_csr_t* A, int32_t K, ns_dtype_t dt, const ns_tune_t* tune,
@@ -243,11 +250,16 @@ void fill_desc(const Plan* P, const void* B, int64_t ldb, float* C, int64_t ldc,
 ns_status_t exec_launch(const ExecDesc* descs, const int32_t* queue, const int32_t* queue_desc,
                         int64_t n_items, int32_t* ctrl, int K, int TM, int TK, bool bf16, bool hint,
                         bool dense, int* grid_cache, cudaStream_t s, const ExecDesc* d0 = nullptr,
-                        int W = 256, int contig = 0);
+                        int W = 256);
 ns_status_t exec_launch_plan(Plan* P, cudaStream_t s);
 ns_status_t exec_prepare(int64_t n_items, int K, int TM, int TK, bool bf16, bool hint, bool dense,
-                         int* grid_out, int W = 256, int contig = 0);
+                         int* grid_out, int W = 256);
 bool plan_contig(const Plan* P);  // contiguous residual stream (tau_tile = inf)
+bool plan_coop(const Plan* P);    // ... with so few chunks that the warps of a CTA share one
+ns_status_t contig_launch(const ExecDesc* descs, const int32_t* queue, const int32_t* queue_desc, int64_t n_items,
+                          int32_t* ctrl, int K, bool bf16, const ContigMode& m, int* grid_cache, cudaStream_t s,
+                          const ExecDesc* d0 = nullptr);
+ns_status_t contig_prepare(int64_t n_items, int K, bool bf16, const ContigMode& m, int* grid_out);
 ns_status_t plan_create(const ns_csr_t* A, int32_t K, ns_dtype_t dt, const ns_tune_t* tune,
                         cudaStream_t s, Plan** out);  // checks + build; on error nothing is kept
 

@@ -1,0 +1,111 @@
+// ns_mem.cuh -- loads and stores with L2 cache policies, shared by the execute kernels.
+#pragma once
+#include <type_traits>
+
+#include "ns_internal.cuh"
+
+namespace ns {
+
+// ---------------------------------------------------------------------------------------------
+// memory helpers with L2 cache policies
+// ---------------------------------------------------------------------------------------------
+struct Policies {
+    uint64_t first, last;
+};
+
+__device__ __forceinline__ Policies make_policies()
+{
+    Policies p;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p.first));
+    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p.last));
+    return p;
+}
+
+template <bool HINT>
+__device__ __forceinline__ int32_t ld_stream_i32(const int32_t* p, uint64_t pol)
+{
+    int32_t v;
+    if (HINT)
+        asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.b32 %0, [%1], %2;"
+                     : "=r"(v) : "l"(p), "l"(pol));
+    else
+        v = __ldg(p);
+    return v;
+}
+
+template <bool HINT>
+__device__ __forceinline__ float ld_stream_f32(const float* p, uint64_t pol)
+{
+    float v;
+    if (HINT)
+        asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.f32 %0, [%1], %2;"
+                     : "=f"(v) : "l"(p), "l"(pol));
+    else
+        v = __ldg(p);
+    return v;
+}
+
+// Four consecutive B elements as loaded: 16 B of FP32 or 8 B of BF16.  Rings of gathers keep
+// this raw form and widen a vector only where it is used: a conversion next to its load would
+// wait for the load there and leave one gather in flight instead of the ring's depth.
+template <bool BF16>
+using BRaw = std::conditional_t<BF16, uint2, float4>;
+
+template <bool BF16, bool HINT>
+__device__ __forceinline__ BRaw<BF16> ld_braw(const void* p, uint64_t pol)
+{
+    BRaw<BF16> r;
+    if constexpr (!BF16) {
+        if (HINT)
+            asm volatile("ld.global.nc.L2::cache_hint.v4.f32 {%0,%1,%2,%3}, [%4], %5;"
+                         : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w) : "l"(p), "l"(pol));
+        else
+            r = __ldg(reinterpret_cast<const float4*>(p));
+    } else {
+        if (HINT)
+            asm volatile("ld.global.nc.L2::cache_hint.v2.b32 {%0,%1}, [%2], %3;"
+                         : "=r"(r.x), "=r"(r.y) : "l"(p), "l"(pol));
+        else
+            r = __ldg(reinterpret_cast<const uint2*>(p));
+    }
+    return r;
+}
+
+template <bool BF16>
+__device__ __forceinline__ BRaw<BF16> braw_zero()
+{
+    if constexpr (BF16) return make_uint2(0u, 0u);
+    else return make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
+__device__ __forceinline__ float4 widen(const float4& v) { return v; }
+__device__ __forceinline__ float4 widen(const uint2& v)  // BF16 is the high half of an FP32
+{
+    return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u),
+                       __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
+}
+
+template <bool HINT>
+__device__ __forceinline__ void st_c4(float* p, float4 v, uint64_t pol)
+{
+    if (HINT)
+        asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1,%2,%3,%4}, %5;"
+                     :: "l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "l"(pol) : "memory");
+    else
+        *reinterpret_cast<float4*>(p) = v;
+}
+
+__device__ __forceinline__ float4 f4_fma(float a, float4 b, float4 c)
+{
+    c.x = fmaf(a, b.x, c.x);
+    c.y = fmaf(a, b.y, c.y);
+    c.z = fmaf(a, b.z, c.z);
+    c.w = fmaf(a, b.w, c.w);
+    return c;
+}
+__device__ __forceinline__ float4 f4_add(float4 a, float4 b)
+{
+    return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
+
+}  // namespace ns

@@ -232,7 +232,9 @@ __global__ void k_chunks(const int32_t* __restrict__ rl_start, const int32_t* __
                 const int64_t i0 = __ldg(rl_rows + k0);
                 if (i0 >= 0 && i0 < m) r.z0 = (int32_t)((int64_t)__ldg(res_rowptr + i0) + (b - __ldg(rl_start + k0)));
             }
-            r.pad0 = r.pad1 = 0;
+            r.flags = (b > (int64_t)__ldg(rl_start + k0) ? kChunkHeadCut : 0) |
+                      (kL >= k0 && (int64_t)__ldg(rl_start + kL + 1) > b1 ? kChunkTailCut : 0);
+            r.pad = 0;
             rec[c] = r;
         }
     }
@@ -788,10 +790,11 @@ ns_status_t plan_build(Plan* P, const ns_csr_t* A, int32_t K, ns_dtype_t dt, con
     {
         Arena a;
         a.reserve(&P->slots, P->st.n_slots * (int64_t)K);
-        a.reserve(&P->split_cnt, P->st.n_split);
+        const int64_t n_cnt = P->st.n_split * contig_slices(K);  // a counter per split row and column slice
+        a.reserve(&P->split_cnt, n_cnt);
         NS_TRY(a.commit(s));
         P->blocks.push_back(a.take());
-        NS_CUDA_TRY(cudaMemsetAsync(P->split_cnt, 0, sizeof(int32_t) * (P->st.n_split > 0 ? P->st.n_split : 1), s));
+        NS_CUDA_TRY(cudaMemsetAsync(P->split_cnt, 0, sizeof(int32_t) * (n_cnt > 0 ? n_cnt : 1), s));
     }
     return NS_OK;
 }

@@ -215,12 +215,18 @@ static int64_t est_plan_bytes(const SGraph& g)
     return (int64_t)g.m * 24 + g.nnz * 8 + 4096;
 }
 
+// arrival counters of a request's split rows, one per column slice
+static size_t cnt_bytes(int64_t n_split, int32_t K)
+{
+    return (size_t)(n_split > 0 ? n_split : 1) * contig_slices(K) * 4;
+}
+
 // a request's own device memory: B, C, the partial-row slots of its plan and their counters
 static int64_t req_bytes(const SGraph& g, int32_t K, ns_dtype_t dt, int64_t n_slots, int64_t n_split)
 {
     const size_t eb = dt == NS_BF16 ? 2 : 4;
     return (int64_t)(al256((size_t)g.n * K * eb) + al256((size_t)g.m * K * 4) + al256((size_t)n_slots * K * 4) +
-                     al256((size_t)(n_split > 0 ? n_split : 1) * 4));
+                     al256(cnt_bytes(n_split, K)));
 }
 
 static void drop_plan(Server* S, SPlan* sp)  // lock held
@@ -470,7 +476,7 @@ static void prepare(Server* S, std::vector<SReq*>& fresh, std::vector<SReq*>& re
         const size_t bB = al256((size_t)g.n * q->r.K * eb);
         const size_t bC = al256((size_t)g.m * q->r.K * 4);
         const size_t bS = al256((size_t)P->st.n_slots * q->r.K * 4);
-        const size_t bN = al256((size_t)(P->st.n_split > 0 ? P->st.n_split : 1) * 4);
+        const size_t bN = al256(cnt_bytes(P->st.n_split, q->r.K));
         void* blk = get_block(S, bB + bC + bS + bN, &q->block_bytes, S->s_copy[q->cls]);
         if (!blk) {
             std::lock_guard<std::mutex> lk(S->mu);
@@ -579,19 +585,27 @@ static void launch_group(Server* S, std::vector<SReq*>& rs, int cls, int K, bool
     cudaEventCreateWithFlags(&L.up_ev, cudaEventDisableTiming);
     cudaEventRecord(L.up_ev, es);
     cudaStreamWaitEvent(es, L.h2d_ev, 0);
+    // every plan of a group has the same form (part of the group's key); B starts on a 256-byte block
+    const bool contig = plan_contig(rs[0]->sp->plan);
+    ContigMode mode;
+    mode.coop = plan_coop(rs[0]->sp->plan);
+    mode.W = S->cfg.tune.chunk_nnz;
     // a bulk launch leaves a quarter of the GPU free, so small requests' launches start at once
     int grid = 0;
     if (cls) {
-        const int contig = 0;
-        if (exec_prepare(ni, K, TM, TK, bf16, S->cfg.tune.l2_hints != 0, dense, &grid, S->cfg.tune.chunk_nnz,
-                         contig) != NS_OK)
-            grid = 0;
+        const ns_status_t pr = contig ? contig_prepare(ni, K, bf16, mode, &grid)
+                                      : exec_prepare(ni, K, TM, TK, bf16, S->cfg.tune.l2_hints != 0, dense, &grid,
+                                                     S->cfg.tune.chunk_nnz);
+        if (pr != NS_OK) grid = 0;
         grid = grid > 4 ? grid * 3 / 4 : grid;
     }
-    ns_status_t r = exec_launch(reinterpret_cast<ExecDesc*>(base), reinterpret_cast<int32_t*>(base + bD),
-                                reinterpret_cast<int32_t*>(base + bD + bQ), ni,
-                                reinterpret_cast<int32_t*>(base + bD + 2 * bQ), K, TM, TK, bf16,
-                                S->cfg.tune.l2_hints != 0, dense, &grid, es, nullptr, S->cfg.tune.chunk_nnz);
+    const ExecDesc* dd = reinterpret_cast<ExecDesc*>(base);
+    int32_t* const dq = reinterpret_cast<int32_t*>(base + bD);
+    int32_t* const dqd = reinterpret_cast<int32_t*>(base + bD + bQ);
+    int32_t* const dctrl = reinterpret_cast<int32_t*>(base + bD + 2 * bQ);
+    ns_status_t r = contig ? contig_launch(dd, dq, dqd, ni, dctrl, K, bf16, mode, &grid, es)
+                           : exec_launch(dd, dq, dqd, ni, dctrl, K, TM, TK, bf16, S->cfg.tune.l2_hints != 0, dense,
+                                         &grid, es, nullptr, S->cfg.tune.chunk_nnz);
     cudaEventCreate(&L.exec_ev);
     cudaEventRecord(L.exec_ev, es);
     const double t_start = serve_clock();
@@ -705,10 +719,12 @@ static void worker_loop(Server* S)
         }
         prepare(S, fresh, ready);
         if (!ready.empty()) {
-            std::map<std::tuple<int, int, int, int, int, int>, std::vector<SReq*>> groups;
+            std::map<std::tuple<int, int, int, int, int, int, int>, std::vector<SReq*>> groups;
             for (SReq* q : ready) {
                 const Plan* P = q->sp->plan;
-                groups[{q->cls, q->r.K, (int)q->r.b_dtype, P->st.n_dwin > 0 ? 1 : 0, P->tune.TM, P->tune.TK}]
+                // kernel form: plans with few chunks take the cooperative form, so they launch apart
+                const int form = plan_contig(P) ? (plan_coop(P) ? 2 : 1) : 0;
+                groups[{q->cls, q->r.K, (int)q->r.b_dtype, P->st.n_dwin > 0 ? 1 : 0, P->tune.TM, P->tune.TK, form}]
                     .push_back(q);
             }
             for (auto& kv : groups)  // small class first
