@@ -136,7 +136,8 @@ class ClockSampler:
 # from one ncu capture (summarised in profiles/), keyed by workload and tune.  It is valid only for
 # the kernel source it was taken on: the digest of the execute kernel's sources must match,
 # otherwise the roofline reports traffic as null.
-EXEC_SOURCES = ("ns_exec.cu", "ns_contig.cu", "ns_mem.cuh", "ns_internal.cuh", "ns_dense.cuh", "ns_dense_tc.cuh", "ns_ptx.cuh")
+EXEC_SOURCES = ("ns_exec.cu", "ns_contig.cu", "ns_exec_f32.cu", "ns_residual.cuh", "ns_mem.cuh",
+                "ns_internal.cuh", "ns_dense.cuh", "ns_dense_tc.cuh", "ns_ptx.cuh")
 MEASURED_TRAFFIC = {
     # (workload, tau_tile, chunk_nnz, l2_hints): (source digest, bytes per launch)
     ("powerlaw", 2147483647, 512, 1): ("ce2d73446f053432", 1676767488 + 542345216),

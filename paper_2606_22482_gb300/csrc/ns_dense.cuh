@@ -132,7 +132,9 @@ __device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo)
     lo = to_tf32(x - __uint_as_float(hi));
 }
 
-template <int L, int VPL, bool BF16, bool HINT>
+template <int NW>
+__device__ void dense_row_meta(const ExecDesc& D, int32_t di, int32_t w, int4* meta);
+template <int L, int VPL, bool BF16, bool HINT, int NW = kExecWarps>
 __device__ void dense_deliver_rows(const ExecDesc& D, int32_t di, int32_t w, float* Cs, int cs_stride,
                                    int4* meta, const Policies& pol);
 
@@ -293,27 +295,19 @@ __device__ void dense_item(const ExecDesc& D, int32_t di, unsigned char* smem, i
             }
         }
     }
+    dense_row_meta<kExecWarps>(D, di, w, meta);
     __syncthreads();
     dense_deliver_rows<L, VPL, BF16, HINT>(D, di, w, Cs, G.cs_stride, meta, pol);
 }
 
-// The window's rows: the tensor-core part (Cs, TM x K FP32 in shared memory) plus the rows'
-// absorbed residual on the CUDA cores, then delivery (stored, or piece 0 of a split row).
-// Latency first: one pass loads every row's id, residual range and split id (a thread per row,
-// into `meta`); then each warp takes its rows (r = warp, warp + 4, ...) and gathers all of their
-// residual nonzeros as one list, 32 entries per load and four B rows in flight, adding them into
-// the rows of Cs it owns; last, the rows are delivered from Cs.
-template <int L, int VPL, bool BF16, bool HINT>
-__device__ void dense_deliver_rows(const ExecDesc& D, int32_t di, int32_t w, float* Cs, int cs_stride,
-                                   int4* meta, const Policies& pol)
+// A dense window's rows, a thread per row: (row id, first residual nonzero, residual length, split id).
+// The caller's next barrier before dense_deliver_rows makes them visible.
+template <int NW>
+__device__ void dense_row_meta(const ExecDesc& D, int32_t di, int32_t w, int4* meta)
 {
-    const int TM = D.TM, K = D.K;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int TM = D.TM;
     const bool absorb = __ldg(D.dwin_absorb + di) != 0;
-    const int nv = K >> 2;
-    const int grp = lane / L, li = lane % L;
-    // ---- row metadata: (row id, first residual nonzero, residual length, split id) ----
-    for (int r = threadIdx.x; r < TM; r += kExecThreads) {
+    for (int r = threadIdx.x; r < TM; r += NW * 32) {
         int32_t i = __ldg(D.win_rows + (int64_t)w * TM + r);
         int32_t z0 = 0, n = 0, sp = -1;
         if (i >= D.m) {  // guard: corrupt plan
@@ -332,12 +326,27 @@ __device__ void dense_deliver_rows(const ExecDesc& D, int32_t di, int32_t w, flo
         }
         meta[r] = make_int4(i, z0, n, sp);
     }
-    __syncthreads();
+}
+
+// The window's rows: the tensor-core part (Cs, TM x K FP32 in shared memory) plus the rows'
+// absorbed residual on the CUDA cores, then delivery (stored, or piece 0 of a split row).
+// The rows' metadata is in `meta` (dense_row_meta, before a barrier); each of the CTA's NW warps
+// takes its rows (r = warp, warp + NW, ...) and gathers all of their
+// residual nonzeros as one list, 32 entries per load and four B rows in flight, adding them into
+// the rows of Cs it owns; last, the rows are delivered from Cs.
+template <int L, int VPL, bool BF16, bool HINT, int NW>
+__device__ void dense_deliver_rows(const ExecDesc& D, int32_t di, int32_t w, float* Cs, int cs_stride,
+                                   int4* meta, const Policies& pol)
+{
+    const int TM = D.TM, K = D.K;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int nv = K >> 2;
+    const int grp = lane / L, li = lane % L;
     // ---- absorbed residual: this warp's rows as one list of nonzeros ----
-    const int nrw = (TM - warp + kExecWarps - 1) / kExecWarps;  // rows warp, warp + 4, ... (<= 16)
+    const int nrw = (TM - warp + NW - 1) / NW;  // rows warp, warp + NW, ... (<= 16)
     int len = 0, z0l = 0;
     if (lane < nrw) {
-        const int4 mt = meta[warp + kExecWarps * lane];
+        const int4 mt = meta[warp + NW * lane];
         len = mt.z;
         z0l = mt.y;
     }
@@ -371,7 +380,7 @@ __device__ void dense_deliver_rows(const ExecDesc& D, int32_t di, int32_t w, flo
                 ec = -1;
             }
         }
-        const int er = warp + kExecWarps * l;  // the entry's row in the window
+        const int er = warp + NW * l;  // the entry's row in the window
         const int cnt = total - e0 < 32 ? total - e0 : 32;
         // the warp gathers the listed B rows, four in flight, lanes across the row
         for (int j0 = 0; j0 < cnt; j0 += 4) {
@@ -411,7 +420,7 @@ __device__ void dense_deliver_rows(const ExecDesc& D, int32_t di, int32_t w, flo
     }
     __syncwarp();
     // ---- delivery, a warp per row ----
-    for (int r = warp; r < TM; r += kExecWarps) {
+    for (int r = warp; r < TM; r += NW) {
         const int4 mt = meta[r];
         const int32_t i = mt.x;
         if (i < 0) continue;

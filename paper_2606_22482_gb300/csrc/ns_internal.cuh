@@ -129,7 +129,8 @@ struct ExecDesc {
     const uint32_t* dtile_bits;
     const int32_t* dtile_voff;
     const void* dtile_vals;
-    const uint16_t* dtile_x;  // BF16 plans: every dense tile expanded, in the tensor-core layout
+    const uint16_t* dtile_x;  // every dense tile expanded, in the tensor-core layout: one plane (BF16
+                              // plans) or the three BF16 pieces of its FP32 values, one after another
     // split rows
     const int32_t* row_split;
     const int32_t* split_np;
@@ -178,7 +179,7 @@ struct Plan {
     uint32_t* dtile_bits = nullptr;
     int32_t* dtile_voff = nullptr;
     void* dtile_vals = nullptr;
-    uint16_t* dtile_x = nullptr;  // BF16 plans: dense tiles expanded (execution format, see k_emit_tiles)
+    uint16_t* dtile_x = nullptr;  // dense tiles expanded: one plane (BF16) or three (FP32); see k_emit_tiles
     const int32_t* res_rowptr = nullptr;  // aliases rowptr when nothing is dense
     const int32_t* res_col = nullptr;
     const float* res_val = nullptr;
@@ -254,6 +255,13 @@ ns_status_t exec_launch(const ExecDesc* descs, const int32_t* queue, const int32
 ns_status_t exec_launch_plan(Plan* P, cudaStream_t s);
 ns_status_t exec_prepare(int64_t n_items, int K, int TM, int TK, bool bf16, bool hint, bool dense,
                          int* grid_out, int W = 256);
+// FP32 plans with dense tiles, launches of up to kF32TcMaxK columns (ns_exec_f32.cu); such a plan
+// keeps its tiles' planes (dtile_x)
+constexpr int kF32TcMaxK = 256;
+ns_status_t f32_prepare(int64_t n_items, int K, int TM, int TK, bool hint, int W, int* grid_out);
+ns_status_t f32_launch(const ExecDesc* descs, const int32_t* queue, const int32_t* queue_desc, int64_t n_items,
+                       int32_t* ctrl, int K, int TM, int TK, bool hint, int W, int* grid_cache, cudaStream_t s,
+                       const ExecDesc* d0);
 bool plan_contig(const Plan* P);  // contiguous residual stream (tau_tile = inf)
 bool plan_coop(const Plan* P);    // ... with so few chunks that the warps of a CTA share one
 ns_status_t contig_launch(const ExecDesc* descs, const int32_t* queue, const int32_t* queue_desc, int64_t n_items,

@@ -108,4 +108,26 @@ __device__ __forceinline__ float4 f4_add(float4 a, float4 b)
     return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
 }
 
+// ---- BF16 pieces of FP32 values ----
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)  // round to nearest even
+{
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+
+// The three BF16 pieces of two values, each pair packed (first value low): x = x0 + x1 + x2 with x0
+// truncated (it never overflows) and x1, x2 rounded to nearest.
+__device__ __forceinline__ void split3(float x, float y, uint32_t& p0, uint32_t& p1, uint32_t& p2)
+{
+    const uint32_t xi = __float_as_uint(x), yi = __float_as_uint(y);
+    p0 = __byte_perm(xi, yi, 0x7632);
+    x -= __uint_as_float(xi & 0xffff0000u);
+    y -= __uint_as_float(yi & 0xffff0000u);
+    p1 = pack_bf16(x, y);
+    x -= __uint_as_float(p1 << 16);
+    y -= __uint_as_float(p1 & 0xffff0000u);
+    p2 = pack_bf16(x, y);
+}
+
 }  // namespace ns

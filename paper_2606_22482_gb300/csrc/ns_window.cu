@@ -16,6 +16,7 @@
 //   W10 residual CSR: every element outside a dense tile, original rows and column order
 // All of it is integer work with fixed orders, matching the CPU reference partition exactly.
 #include "ns_internal.cuh"
+#include "ns_mem.cuh"
 #include "ns_scan.cuh"
 
 #include <cuda_bf16.h>
@@ -661,7 +662,9 @@ struct EmitArgs {
     int32_t cap_tiles;
     int32_t tk_log;     // log2(TK)
     uint16_t* dtile_x;  // BF16 plans: the values go straight into the expanded tiles (zeroed
-                        // beforehand) and k_pack_tiles packs them afterwards; NULL: packed here
+                        // beforehand) and k_pack_tiles packs them afterwards; NULL: see dtile_f
+    float* dtile_f;     // FP32 plans with K <= 256: likewise, expanded FP32 tiles (a temporary) that
+                        // k_pack_tiles_f32 packs and splits; both NULL: packed here
 };
 
 // Position of element (row r, compacted column c) inside an expanded TM x TK tile: 8 x 8 blocks
@@ -695,6 +698,7 @@ __global__ void __launch_bounds__(kWinThreads, 4) k_emit_tiles(EmitArgs a)
     const int64_t ntile = (U + TK - 1) / TK;
     const int32_t dbase = a.win_dptr[w];
     const int32_t ndt = a.win_ndt[w];
+    const bool expand = a.dtile_x || a.dtile_f;
     // the window's dense-tile bitmaps (and tile ranks) in shared memory when they fit, else the
     // plan's bitmaps with global atomics and the ranks from global memory
     const bool in_smem = (int64_t)ndt * BW <= a.cap_words && ntile <= a.cap_tiles;
@@ -729,7 +733,7 @@ __global__ void __launch_bounds__(kWinThreads, 4) k_emit_tiles(EmitArgs a)
             for (int u = 0; u < 4; ++u) {
                 const int64_t e = eb + 32 * u + lane;
                 pv[u] = e < rend ? a.epos[wbase + e] : -1;
-                if (a.dtile_x) iv[u] = e < rend ? (a.eidx ? a.eidx[wbase + e] : (int32_t)(wbase + e)) : -1;
+                if (expand) iv[u] = e < rend ? (a.eidx ? a.eidx[wbase + e] : (int32_t)(wbase + e)) : -1;
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -744,11 +748,15 @@ __global__ void __launch_bounds__(kWinThreads, 4) k_emit_tiles(EmitArgs a)
                         const int bit = (r << tkl) + (pv[u] & (TK - 1));
                         key = k * BW + (bit >> 5);
                         mbit = 1u << (bit & 31);
-                        if (a.dtile_x) {  // BF16: the value into its expanded tile
+                        if (expand) {  // the value into its expanded tile
                             const float v = __ldg(a.vals + iv[u]);
-                            __nv_bfloat16 h = __float2bfloat16_rn(v);
-                            a.dtile_x[(int64_t)(dbase + k) * TM * TK + tile_x_offset(r, pv[u] & (TK - 1), TK)] =
-                                *reinterpret_cast<uint16_t*>(&h);
+                            const int64_t at = (int64_t)(dbase + k) * TM * TK + tile_x_offset(r, pv[u] & (TK - 1), TK);
+                            if (a.dtile_f) {
+                                a.dtile_f[at] = v;
+                            } else {
+                                __nv_bfloat16 h = __float2bfloat16_rn(v);
+                                a.dtile_x[at] = *reinterpret_cast<uint16_t*>(&h);
+                            }
                             a.pdense[iv[u]] = 1;
                         }
                     }
@@ -768,7 +776,7 @@ __global__ void __launch_bounds__(kWinThreads, 4) k_emit_tiles(EmitArgs a)
         }
     }
     __syncthreads();
-    if (a.dtile_x) {  // BF16: values already placed; k_pack_tiles packs them from the tiles
+    if (expand) {  // values already placed; they are packed from the tiles
         if (in_smem)
             for (int q = threadIdx.x; q < ndt * BW; q += blockDim.x) a.dtile_bits[(int64_t)dbase * BW + q] = sbits[q];
         return;
@@ -832,13 +840,14 @@ __global__ void __launch_bounds__(kWinThreads, 4) k_emit_tiles(EmitArgs a)
     }
 }
 
-// W9b: BF16 plans, packed values from the expanded tiles (emission wrote each value straight into
+// W9b: packed values from the expanded tiles (emission wrote each value straight into
 // its tile at tile_x_offset).  One warp per tile: the lanes take the bitmap's words in order, 32
 // bits at a time; a set bit's value goes to its rank in bitmap order (the words' popcounts scanned
 // across the lanes, plus the bits before it in its word).
+template <class V>
 __global__ void k_pack_tiles(const uint32_t* __restrict__ bits, const int32_t* __restrict__ voff,
-                             const uint16_t* __restrict__ x, int64_t n_dtiles, int32_t TM, int32_t TK,
-                             uint16_t* __restrict__ vals)
+                             const V* __restrict__ x, int64_t n_dtiles, int32_t TM, int32_t TK,
+                             V* __restrict__ vals)
 {
     const int lane = threadIdx.x & 31;
     const int BW = TM * TK / 32;
@@ -862,7 +871,7 @@ __global__ void k_pack_tiles(const uint32_t* __restrict__ bits, const int32_t* _
         }
         const int excl = incl - own;
         const int64_t v0 = __ldg(voff + d);
-        const uint16_t* tx = x + d * (int64_t)TM * TK;
+        const V* tx = x + d * (int64_t)TM * TK;
 #pragma unroll 8
         for (int q = 0; q < BW; ++q) {
             const int src = WPL == 2 ? q >> 1 : q, j = WPL == 2 ? q & 1 : 0;
@@ -874,6 +883,25 @@ __global__ void k_pack_tiles(const uint32_t* __restrict__ bits, const int32_t* _
                 vals[v0 + base + __popc(word & ((1u << lane) - 1u))] = tx[tile_x_offset(b >> tkl, b & (TK - 1), TK)];
             }
         }
+    }
+}
+
+// W9c: FP32 plans, the three BF16 planes of every expanded tile (x = x0 + x1 + x2: x0 truncated, so
+// that it never overflows, x1 and x2 rounded to nearest), plane after plane in each tile, all in the
+// layout of tile_x_offset.  A thread splits eight consecutive elements: 32 bytes in, three times 16
+// bytes out, all coalesced.
+__global__ void k_split_tiles(const float* __restrict__ x, int64_t n_eights, int32_t eights, uint16_t* __restrict__ planes)
+{
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n_eights; q += (int64_t)gridDim.x * blockDim.x) {
+        const float4 a = __ldg(reinterpret_cast<const float4*>(x) + 2 * q), b = __ldg(reinterpret_cast<const float4*>(x) + 2 * q + 1);
+        const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+        uint32_t p[3][4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) split3(v[2 * e], v[2 * e + 1], p[0][e], p[1][e], p[2][e]);
+        const int64_t tile = q / eights;
+        uint4* out = reinterpret_cast<uint4*>(planes) + tile * 3 * eights + (q - tile * eights);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) out[(int64_t)k * eights] = make_uint4(p[k][0], p[k][1], p[k][2], p[k][3]);
     }
 }
 
@@ -1278,7 +1306,17 @@ ns_status_t window_pass(Plan* P, WindowResult* W, cudaStream_t s)
     pb.reserve_bytes(&P->dtile_vals, (size_t)(n_dvals > 0 ? n_dvals : 1) * (bf16 ? 2 : 4));
     pb.reserve(&P->res_col_own, n_res);
     pb.reserve(&P->res_val_own, n_res);
+    // FP32: planes for the launches of up to kF32TcMaxK columns (the whole width, or a column slice)
+    const int32_t K = P->K, TN = t.TN > 0 && t.TN < K ? t.TN : K;
+    const bool planes = !bf16 && (TN <= kF32TcMaxK || (K % TN != 0 && K % TN <= kF32TcMaxK));
+    float* dtile_f = nullptr;
+    Arena tf;  // temporary
+    if (planes && n_dtiles > 0) {
+        tf.reserve(&dtile_f, n_dtiles * TM * TK);
+        NS_TRY(tf.commit(s));
+    }
     if (bf16) pb.reserve(&P->dtile_x, n_dtiles * TM * TK);
+    if (planes) pb.reserve(&P->dtile_x, 3 * n_dtiles * TM * TK);
     NS_TRY(pb.commit(s));
     P->blocks.push_back(pb.take());
     P->res_col = P->res_col_own;
@@ -1305,17 +1343,26 @@ ns_status_t window_pass(Plan* P, WindowResult* W, cudaStream_t s)
         EmitArgs ea{row_kbase, eidx, epos, ucan, trank, tvoff, win_U, win_ndt, P->win_dptr, win_vbase,
                     P->vals, m_aic, TM, TK, bf16 ? 1 : 0, P->dtile_cols, P->dtile_bits, P->dtile_voff,
                     P->dtile_vals, pdense, (int32_t)cap_words, (int32_t)cap_tiles, ilog2(TK),
-                    bf16 ? P->dtile_x : nullptr};
+                    bf16 ? P->dtile_x : nullptr, dtile_f};
         if (bf16) NS_CUDA_TRY(cudaMemsetAsync(P->dtile_x, 0, sizeof(uint16_t) * n_dtiles * TM * TK, s));
+        if (dtile_f) NS_CUDA_TRY(cudaMemsetAsync(dtile_f, 0, sizeof(float) * n_dtiles * TM * TK, s));
         k_emit_tiles<<<(unsigned)n_win, kWinThreads, dyn, s>>>(ea);
         NS_LAUNCH_CHECK();
+        const int64_t blocks64 = (n_dtiles * 32 + 255) / 256;
+        const unsigned blocks = (unsigned)(blocks64 < 65535 * 8 ? blocks64 : 65535 * 8);
         if (bf16) {
-            const int64_t warps = n_dtiles;
-            const int64_t blocks = (warps * 32 + 255) / 256;
-            k_pack_tiles<<<(unsigned)(blocks < 65535 * 8 ? blocks : 65535 * 8), 256, 0, s>>>(
-                P->dtile_bits, P->dtile_voff, P->dtile_x, n_dtiles, TM, TK,
-                reinterpret_cast<uint16_t*>(P->dtile_vals));
+            k_pack_tiles<uint16_t><<<blocks, 256, 0, s>>>(P->dtile_bits, P->dtile_voff, P->dtile_x, n_dtiles, TM, TK,
+                                                          reinterpret_cast<uint16_t*>(P->dtile_vals));
             NS_LAUNCH_CHECK();
+        }
+        if (dtile_f) {
+            k_pack_tiles<float><<<blocks, 256, 0, s>>>(P->dtile_bits, P->dtile_voff, dtile_f, n_dtiles, TM, TK,
+                                                       reinterpret_cast<float*>(P->dtile_vals));
+            NS_LAUNCH_CHECK();
+            const int64_t eights = TM * TK / 8;
+            k_split_tiles<<<wgrid(n_dtiles * eights), 256, 0, s>>>(dtile_f, n_dtiles * eights, (int32_t)eights, P->dtile_x);
+            NS_LAUNCH_CHECK();
+            tf.release(s);
         }
     }
     if (m > 0) {
