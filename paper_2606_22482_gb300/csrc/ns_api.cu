@@ -106,30 +106,15 @@ void Arena::release(cudaStream_t s)
     reqs.clear();
 }
 
-// Stream-ordered release: the blocks go back to the pool after everything already enqueued on
-// the stream of the last plan/execute call, so a destroy right after an asynchronous execute
-// never frees memory a running kernel still reads.
-Plan::~Plan()
-{
-    if (status_ev) cudaEventDestroy(status_ev);
-    bool failed = false;
-    for (auto& b : blocks) {
-        if (!b.ptr) continue;
-        if (!failed && cudaFreeAsync(b.ptr, last_stream) != cudaSuccess) {
-            (void)cudaGetLastError();
-            failed = true;
-            cudaDeviceSynchronize();
-        }
-        if (failed) cudaFree(b.ptr);
-        b.ptr = nullptr;
-    }
-}
-
-// pinned host slots for the status words of plans (one slab for the process)
+// Pinned host slots for the status words of plans (one slab for the process).  A live plan has a slot
+// of its own: its launches write there, and nothing but the plan's own word may be read from it.  Slots
+// are handed out in turn, so a freed one comes back as late as possible; with every slot taken, two
+// plans share one.
 static std::mutex g_slab_mu;
 static int32_t* g_slab = nullptr;
 static uint32_t g_slab_next = 0;
 constexpr uint32_t kSlabSlots = 65536;
+static uint32_t g_slab_users[kSlabSlots];
 
 static int32_t* status_slot()
 {
@@ -142,9 +127,35 @@ static int32_t* status_slot()
         }
         memset(g_slab, 0, kSlabSlots * sizeof(int32_t));
     }
-    int32_t* p = g_slab + (g_slab_next++ % kSlabSlots);
-    *p = 0;
-    return p;
+    for (uint32_t k = 0; k < kSlabSlots && g_slab_users[g_slab_next % kSlabSlots]; ++k) ++g_slab_next;
+    const uint32_t i = g_slab_next++ % kSlabSlots;
+    if (!g_slab_users[i]++) g_slab[i] = 0;
+    return g_slab + i;
+}
+
+static void status_give(volatile int32_t* slot)
+{
+    std::lock_guard<std::mutex> lk(g_slab_mu);
+    --g_slab_users[slot - g_slab];
+}
+
+// Stream-ordered release: the blocks go back to the pool after everything already enqueued on
+// the stream of the last plan/execute call, so a destroy right after an asynchronous execute
+// never frees memory a running kernel still reads.
+Plan::~Plan()
+{
+    if (status_host) status_give(status_host);
+    bool failed = false;
+    for (auto& b : blocks) {
+        if (!b.ptr) continue;
+        if (!failed && cudaFreeAsync(b.ptr, last_stream) != cudaSuccess) {
+            (void)cudaGetLastError();
+            failed = true;
+            cudaDeviceSynchronize();
+        }
+        if (failed) cudaFree(b.ptr);
+        b.ptr = nullptr;
+    }
 }
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -210,6 +221,16 @@ ns_status_t plan_create(const ns_csr_t* A, int32_t K, ns_dtype_t b_dtype, const 
         (void)cudaGetLastError();
         delete P;
         return r;
+    }
+    if (int32_t* slot = status_slot()) {
+        void* map = nullptr;
+        if (cudaHostGetDevicePointer(&map, slot, 0) == cudaSuccess) {
+            P->status_host = slot;
+            P->status_map = static_cast<int32_t*>(map);
+        } else {
+            status_give(slot);
+            (void)cudaGetLastError();
+        }
     }
     P->st.device_bytes = 0;
     for (auto& b : P->blocks) P->st.device_bytes += (int64_t)b.bytes;
@@ -331,9 +352,9 @@ ns_status_t ns_spmm_execute(ns_plan_t p, const void* B, int64_t ldb, float* C, i
         cudaEventDestroy(ev);
         P->last_stream = st;
     }
-    // the device status word of an earlier launch, if its pinned copy has already landed
+    // the status word an earlier launch has reported, if any
     // (never waits: a launch still running is checked by a later call)
-    if (P->status_ev && cudaEventQuery(P->status_ev) == cudaSuccess) {
+    if (P->status_host) {
         const int32_t status = *P->status_host;
         if (status & kStatusTimeout) {
             set_error("an earlier launch gave up a bounded wait");
@@ -356,14 +377,8 @@ ns_status_t ns_spmm_execute(ns_plan_t p, const void* B, int64_t ldb, float* C, i
         P->desc_valid = true;
         NS_TRY(exec_launch_plan(P, st));
     }
-    if (!P->status_host) {
-        P->status_host = status_slot();
-        if (P->status_host) cudaEventCreateWithFlags(&P->status_ev, cudaEventDisableTiming);
-    }
-    if (P->status_host && P->status_ev) {
-        cudaMemcpyAsync(P->status_host, P->ctrl + 2, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
-        cudaEventRecord(P->status_ev, st);
-    }
+    if (P->st.n_items == 0 && P->status_map)  // nothing was launched that could report
+        cudaMemcpyAsync(P->status_map, P->ctrl + 2, sizeof(int32_t), cudaMemcpyDefault, st);
     return NS_OK;
 }
 

@@ -533,16 +533,7 @@ __global__ void __launch_bounds__(kExecThreads, FORM == kFormBf16 ? 6 : (G == 16
         }
         u = first + (int64_t)next;
     }
-    // the last CTA out resets the tickets for the next launch (stream order makes it visible)
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const int done = atomicAdd(ctrl + 1, 1);
-        if (done == (int)gridDim.x - 1) {
-            atomicExch(ticket, 0ull);
-            atomicExch(ctrl + 1, 0);
-        }
-    }
+    end_launch(ctrl, d0, descs == nullptr);
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(kExecThreads, DENSE ? 1 : 4) k_exec(const Exec
     // phase 2: residual chunks
     residual_phase<L, VPL, BF16, HINT>(descs, queue, queue_desc, n_items, ctrl, d0, lane, warp, smem_raw, kExecWarps,
                                        pol, clk);
-    reset_tickets(ctrl);
+    end_launch(ctrl, d0, descs == nullptr);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -157,6 +157,7 @@ void fill_desc(const Plan* P, const void* B, int64_t ldb, float* C, int64_t ldc,
     d->hot = P->hot_bits;
     d->chunk_nnz = P->tune.chunk_nnz;
     d->status = P->ctrl + 2;
+    d->status_out = P->status_map;
     d->class_clock = P->class_clock;
 }
 

@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(kTsThreads, 1) k_exec_f32(const ExecDesc* __re
     if (warp < res_warps)
         residual_phase<32, VPL, false, HINT>(descs, queue, queue_desc, n_items, ctrl, d0, lane, warp, smem_raw, res_warps,
                                              pol, clk);
-    reset_tickets(ctrl);
+    end_launch(ctrl, d0, descs == nullptr);
 }
 
 // ---------------------------------------------------------------------------------------------

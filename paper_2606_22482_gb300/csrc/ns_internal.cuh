@@ -149,6 +149,7 @@ struct ExecDesc {
     const uint32_t* hot;   // bit j set: B row j is among the most gathered (evict-last); null: all
     int32_t chunk_nnz;     // W of the plan (sizes the staged chunk buffers)
     int32_t* status;       // device status word (kStatus* bits)
+    int32_t* status_out;   // mapped host word the launch's last CTA copies a nonzero status to, or null
     // per-class progress clock (Section 5.3 epoch monitoring), null when off: [0] earliest CTA
     // start, [1] latest end of a dense item, [2] latest end of a residual chunk (globaltimer ns)
     unsigned long long* class_clock;
@@ -210,8 +211,8 @@ struct Plan {
     int exec_grid = 0;
     int exec_grid_slice = 0, exec_grid_slice_K = 0;  // grid of the column-slice launches
     cudaStream_t last_stream = nullptr;  // stream of the last plan/execute call: frees go there
-    int32_t* status_host = nullptr;      // pinned copy of the device status word after a launch
-    cudaEvent_t status_ev = nullptr;     // completes when that copy has landed
+    volatile int32_t* status_host = nullptr;  // mapped host word: the status a finished launch reported
+    int32_t* status_map = nullptr;            // its device address
     ~Plan();
 };
 

@@ -130,4 +130,27 @@ __device__ __forceinline__ void split3(float x, float y, uint32_t& p0, uint32_t&
     p2 = pack_bf16(x, y);
 }
 
+// The end of a persistent launch, called by the whole CTA: the last CTA out resets the tickets for the
+// next launch (stream order makes it visible) and reports a nonzero status word to the host.  A
+// copy and an event after every launch did that before, two calls and a copy engine's turn: 13.5 ->
+// 9.2 us for an execute of 65 536 nonzeros at K = 32, 110.5 -> 105.1 us for the attention mask's.
+__device__ __forceinline__ void end_launch(int32_t* ctrl, const ExecDesc& d0, bool single)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        const int done = atomicAdd(ctrl + 1, 1);
+        if (done == (int)gridDim.x - 1) {
+            atomicExch(ctrl + 0, 0);
+            atomicExch(ctrl + 3, 0);
+            atomicExch(reinterpret_cast<unsigned long long*>(ctrl + 4), 0ull);
+            atomicExch(ctrl + 1, 0);
+            if (single && d0.status_out) {
+                const int32_t st = atomicOr(d0.status, 0);
+                if (st) *reinterpret_cast<volatile int32_t*>(d0.status_out) = st;
+            }
+        }
+    }
+}
+
 }  // namespace ns

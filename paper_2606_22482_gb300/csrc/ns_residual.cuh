@@ -520,20 +520,4 @@ __device__ __forceinline__ void residual_phase(const ExecDesc* descs, const int3
     }
 }
 
-// the last CTA out resets the tickets for the next launch (stream order makes it visible); called
-// by the whole CTA
-__device__ __forceinline__ void reset_tickets(int32_t* ctrl)
-{
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        int done = atomicAdd(ctrl + 1, 1);
-        if (done == (int)gridDim.x - 1) {
-            atomicExch(ctrl + 0, 0);
-            atomicExch(ctrl + 3, 0);
-            atomicExch(ctrl + 1, 0);
-        }
-    }
-}
-
 }  // namespace ns
