@@ -21,6 +21,8 @@
 
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 namespace ns {
 
 constexpr int kWinThreads = 512;
@@ -43,6 +45,8 @@ constexpr size_t count_table_bytes(int64_t n)
 // (2 bytes a word) and its tiles' dense ranks (2 bytes a tile) in dynamic shared memory sized
 // from the plan's largest window, up to this limit (larger windows use global memory)
 constexpr int kEmitSmemMax = 192 * 1024;
+// tile ranks of a window in shared memory (no opt-in needed)
+constexpr int kPlaceSmemMax = 40 * 1024;
 
 // ---------------------------------------------------------------------------------------------
 // W1: kept rows
@@ -599,16 +603,19 @@ __global__ void k_dense_windows(const int32_t* __restrict__ dwin, int64_t n_dwin
                                 int32_t TK, int32_t absorb_cap, int64_t cost_tc, int64_t cost_res,
                                 int32_t* dwin_absorb, int64_t* dcost, int8_t* row_state)
 {
-    for (int64_t d = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; d < n_dwin;
-         d += (int64_t)gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31;  // a warp per window
+    for (int64_t d = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; d < n_dwin;
+         d += ((int64_t)gridDim.x * blockDim.x) >> 5) {
         int32_t w = dwin[d];
         int64_t r0 = (int64_t)w * TM;
         int64_t nvalid = m_aic - r0 < TM ? m_aic - r0 : TM;
         int64_t res = win_res[w];
         int absorb = res <= absorb_cap;
-        dwin_absorb[d] = absorb;
-        dcost[d] = (int64_t)win_ndt[w] * TM * TK * cost_tc + ((absorb ? res : 0) + nvalid) * cost_res;
-        for (int64_t r = 0; r < nvalid; ++r) row_state[aic_rows[r0 + r]] = absorb ? 1 : 2;
+        if (lane == 0) {
+            dwin_absorb[d] = absorb;
+            dcost[d] = (int64_t)win_ndt[w] * TM * TK * cost_tc + ((absorb ? res : 0) + nvalid) * cost_res;
+        }
+        for (int64_t r = lane; r < nvalid; r += 32) row_state[aic_rows[r0 + r]] = absorb ? 1 : 2;
     }
 }
 
@@ -637,7 +644,7 @@ struct RlStore {
 };
 
 // ---------------------------------------------------------------------------------------------
-// W9: emit dense tiles (one CTA per window)
+// W9: emit dense tiles (one CTA per window) of plans without expanded tiles (FP32, K > kF32TcMaxK)
 // ---------------------------------------------------------------------------------------------
 struct EmitArgs {
     const int64_t* row_kbase;
@@ -652,19 +659,15 @@ struct EmitArgs {
     const int64_t* win_vbase;
     const float* vals;
     int64_t m_aic;
-    int32_t TM, TK, bf16;
+    int32_t TM, TK;
     int32_t* dtile_cols;
     uint32_t* dtile_bits;
     int32_t* dtile_voff;
-    void* dtile_vals;
+    float* dtile_vals;
     uint8_t* pdense;  // per original element: 1 if in a dense tile
     int32_t cap_words;  // bitmap words and tiles a window may have for the shared-memory path
     int32_t cap_tiles;
     int32_t tk_log;     // log2(TK)
-    uint16_t* dtile_x;  // BF16 plans: the values go straight into the expanded tiles (zeroed
-                        // beforehand) and k_pack_tiles packs them afterwards; NULL: see dtile_f
-    float* dtile_f;     // FP32 plans with K <= 256: likewise, expanded FP32 tiles (a temporary) that
-                        // k_pack_tiles_f32 packs and splits; both NULL: packed here
 };
 
 // Position of element (row r, compacted column c) inside an expanded TM x TK tile: 8 x 8 blocks
@@ -698,7 +701,6 @@ __global__ void __launch_bounds__(kWinThreads, 4) k_emit_tiles(EmitArgs a)
     const int64_t ntile = (U + TK - 1) / TK;
     const int32_t dbase = a.win_dptr[w];
     const int32_t ndt = a.win_ndt[w];
-    const bool expand = a.dtile_x || a.dtile_f;
     // the window's dense-tile bitmaps (and tile ranks) in shared memory when they fit, else the
     // plan's bitmaps with global atomics and the ranks from global memory
     const bool in_smem = (int64_t)ndt * BW <= a.cap_words && ntile <= a.cap_tiles;
@@ -733,7 +735,6 @@ __global__ void __launch_bounds__(kWinThreads, 4) k_emit_tiles(EmitArgs a)
             for (int u = 0; u < 4; ++u) {
                 const int64_t e = eb + 32 * u + lane;
                 pv[u] = e < rend ? a.epos[wbase + e] : -1;
-                if (expand) iv[u] = e < rend ? (a.eidx ? a.eidx[wbase + e] : (int32_t)(wbase + e)) : -1;
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -748,17 +749,6 @@ __global__ void __launch_bounds__(kWinThreads, 4) k_emit_tiles(EmitArgs a)
                         const int bit = (r << tkl) + (pv[u] & (TK - 1));
                         key = k * BW + (bit >> 5);
                         mbit = 1u << (bit & 31);
-                        if (expand) {  // the value into its expanded tile
-                            const float v = __ldg(a.vals + iv[u]);
-                            const int64_t at = (int64_t)(dbase + k) * TM * TK + tile_x_offset(r, pv[u] & (TK - 1), TK);
-                            if (a.dtile_f) {
-                                a.dtile_f[at] = v;
-                            } else {
-                                __nv_bfloat16 h = __float2bfloat16_rn(v);
-                                a.dtile_x[at] = *reinterpret_cast<uint16_t*>(&h);
-                            }
-                            a.pdense[iv[u]] = 1;
-                        }
                     }
                 }
 #pragma unroll
@@ -776,11 +766,6 @@ __global__ void __launch_bounds__(kWinThreads, 4) k_emit_tiles(EmitArgs a)
         }
     }
     __syncthreads();
-    if (expand) {  // values already placed; they are packed from the tiles
-        if (in_smem)
-            for (int q = threadIdx.x; q < ndt * BW; q += blockDim.x) a.dtile_bits[(int64_t)dbase * BW + q] = sbits[q];
-        return;
-    }
     // per dense tile, the value index of each bitmap word's first bit
     if (in_smem) {
         for (int q = threadIdx.x; q < ndt * BW; q += blockDim.x) a.dtile_bits[(int64_t)dbase * BW + q] = sbits[q];
@@ -827,62 +812,172 @@ __global__ void __launch_bounds__(kWinThreads, 4) k_emit_tiles(EmitArgs a)
             }
             const int64_t vi = vbase + tv + idx;
             const float v = __ldg(a.vals + p);
-            if (a.bf16) {
-                __nv_bfloat16 h = __float2bfloat16_rn(v);
-                const uint16_t hb = *reinterpret_cast<uint16_t*>(&h);
-                reinterpret_cast<uint16_t*>(a.dtile_vals)[vi] = hb;
-            } else {
-                reinterpret_cast<float*>(a.dtile_vals)[vi] = v;
-            }
+            a.dtile_vals[vi] = v;
             a.pdense[p] = 1;
           }
         }
     }
 }
 
-// W9b: packed values from the expanded tiles (emission wrote each value straight into
-// its tile at tile_x_offset).  One warp per tile: the lanes take the bitmap's words in order, 32
-// bits at a time; a set bit's value goes to its rank in bitmap order (the words' popcounts scanned
-// across the lanes, plus the bits before it in its word).
+// W9a: plans that keep expanded tiles (BF16, and FP32 up to kF32TcMaxK columns): each value goes
+// straight to its place in its window's expanded tiles (filled with kNoValue beforehand), one warp
+// per row.  Where the windows hold all of A in CSR order (`ident`), the same pass writes the residual
+// CSR: the row's other elements in order.  Assembling the bitmaps here as well (a segmented OR over
+// the warp and a shared atomic per run), marking dense elements in a byte array and leaving the
+// residual to a pass of its own took 326 + 49 us on the attention mask (32 768 rows, TM 64, TK 32);
+// this takes 291, and planning with one execute 1120 -> 955 us.
 template <class V>
-__global__ void k_pack_tiles(const uint32_t* __restrict__ bits, const int32_t* __restrict__ voff,
-                             const V* __restrict__ x, int64_t n_dtiles, int32_t TM, int32_t TK,
-                             V* __restrict__ vals)
+struct PlaceArgs {
+    const int64_t* row_kbase;
+    const int32_t* eidx;  // CSR position of each window element; NULL (ident): element e is position e
+    const int32_t* epos;
+    const int32_t* ucan;
+    const int32_t* trank;
+    const int32_t* tvoff;
+    const int32_t* win_U;
+    const int32_t* win_ndt;
+    const int32_t* win_dptr;
+    const int64_t* win_vbase;
+    const float* vals;
+    int64_t m_aic;
+    int32_t TM, TK;
+    int32_t* dtile_cols;
+    int32_t* dtile_voff;
+    V* tiles;
+    uint8_t* pdense;            // !ident: per original element, 1 if in a dense tile
+    const int32_t* colidx;      // ident: the residual CSR
+    const int32_t* res_rowptr;
+    int32_t* res_col;
+    float* res_val;
+    int32_t cap_tiles;          // tile ranks kept in shared memory
+    int32_t tk_log;
+};
+
+// No value of a tile has these bits: the BF16 cast gives NaNs another pattern, and an FP32 NaN of all
+// ones is stored as the NaN next to it.
+template <class V>
+struct TileValue;
+template <>
+struct TileValue<uint16_t> {
+    static __device__ __forceinline__ uint16_t of(float v) { return __bfloat16_as_ushort(__float2bfloat16_rn(v)); }
+    static __device__ __forceinline__ bool none(uint16_t h) { return h == 0xffffu; }
+};
+template <>
+struct TileValue<float> {
+    static __device__ __forceinline__ float of(float v) { return none(v) ? __uint_as_float(0xfffffffeu) : v; }
+    static __device__ __forceinline__ bool none(float v) { return __float_as_uint(v) == 0xffffffffu; }
+};
+
+template <class V>
+__global__ void __launch_bounds__(kWinThreads, 3) k_place_tiles(PlaceArgs<V> a)
+{
+    __shared__ int64_t rb0[kMaxTM + 1];
+    extern __shared__ int16_t place_rank[];
+    const int tkl = a.tk_log, TM = a.TM, TK = a.TK;
+    const int w = blockIdx.x;
+    const bool ident = a.eidx == nullptr;
+    const int32_t ndt = a.win_ndt[w];
+    if (ndt == 0 && !ident) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int64_t r0 = (int64_t)w * TM;
+    const int nrows = (int)(a.m_aic - r0 < TM ? a.m_aic - r0 : TM);
+    const int64_t wbase = a.row_kbase[r0];
+    for (int q = threadIdx.x; q <= nrows; q += blockDim.x) rb0[q] = a.row_kbase[r0 + q] - wbase;
+    const int64_t U = a.win_U[w];
+    const int64_t ntile = (U + TK - 1) / TK;
+    const int32_t dbase = a.win_dptr[w];
+    const bool in_smem = ntile <= a.cap_tiles;
+    for (int64_t t = threadIdx.x; t < ntile; t += blockDim.x) {
+        const int32_t k = a.trank[wbase + t];
+        if (in_smem) place_rank[t] = (int16_t)k;
+        if (k >= 0) a.dtile_voff[dbase + k] = (int32_t)(a.win_vbase[w] + a.tvoff[wbase + t]);
+    }
+    // columns of the dense tiles: one thread per (tile, column), reads of ucan coalesced
+    for (int64_t q = threadIdx.x; q < ntile * TK; q += blockDim.x) {
+        const int32_t k = a.trank[wbase + (q >> tkl)];
+        if (k >= 0) a.dtile_cols[(int64_t)(dbase + k) * TK + (q & (TK - 1))] = q < U ? a.ucan[wbase + q] : -1;
+    }
+    __syncthreads();
+    V* const tiles = a.tiles + (int64_t)dbase * TM * TK;
+    for (int r = warp; r < nrows; r += nwarps) {
+        const int64_t rend = rb0[r + 1];
+        V* const trow = tiles + tile_x_offset(r, 0, TK);
+        int64_t out = ident ? a.res_rowptr[r0 + r] : 0;
+        for (int64_t eb = rb0[r]; eb < rend; eb += 128) {  // four elements per lane in flight
+            int32_t pv[4], iv[4];
+            float vv[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t e = eb + 32 * u + lane;
+                pv[u] = e < rend ? a.epos[wbase + e] : -1;
+                iv[u] = e < rend ? (ident ? (int32_t)(wbase + e) : a.eidx[wbase + e]) : 0;
+                vv[u] = e < rend ? __ldg(a.vals + iv[u]) : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int32_t pos = pv[u];
+                int32_t k = -1;
+                if (pos >= 0) k = in_smem ? (int32_t)place_rank[pos >> tkl] : a.trank[wbase + (pos >> tkl)];
+                if (k >= 0) {
+                    const int c = pos & (TK - 1);
+                    trow[(int64_t)k * TM * TK + (c >> 3) * 64 + (c & 7)] = TileValue<V>::of(vv[u]);
+                    if (!ident) a.pdense[iv[u]] = 1;
+                }
+                if (ident) {
+                    const bool keep = pos >= 0 && k < 0;
+                    const unsigned bal = __ballot_sync(0xffffffffu, keep);
+                    if (keep) {
+                        const int64_t o = out + __popc(bal & ((1u << lane) - 1u));
+                        a.res_col[o] = __ldg(a.colidx + iv[u]);
+                        a.res_val[o] = vv[u];
+                    }
+                    out += __popc(bal);
+                }
+            }
+        }
+    }
+}
+
+// W9b: bitmaps and packed values from the expanded tiles, one warp per tile: 32 elements of the tile at
+// a time in bitmap order; a present value goes to its rank.  BF16 tiles are what the execute kernel
+// multiplies, so their absent places become zeros.  Values are padded to a multiple of 8 with zeros.
+template <class V>
+__global__ void k_pack_tiles(V* __restrict__ x, const int32_t* __restrict__ voff, int64_t n_dtiles, int32_t TM,
+                             int32_t TK, uint32_t* __restrict__ bits, V* __restrict__ vals)
 {
     const int lane = threadIdx.x & 31;
     const int BW = TM * TK / 32;
-    const int WPL = (BW + 31) / 32;
     const int tkl = TK == 32 ? 5 : 4;
     for (int64_t d = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; d < n_dtiles;
          d += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-        const uint32_t* tb = bits + d * BW;
-        uint32_t wv[2] = {0u, 0u};
-        int own = 0;
-        for (int j = 0; j < WPL; ++j) {
-            const int q = lane * WPL + j;
-            wv[j] = q < BW ? __ldg(tb + q) : 0u;
-            own += __popc(wv[j]);
-        }
-        int incl = own;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        const int excl = incl - own;
         const int64_t v0 = __ldg(voff + d);
-        const V* tx = x + d * (int64_t)TM * TK;
-#pragma unroll 8
-        for (int q = 0; q < BW; ++q) {
-            const int src = WPL == 2 ? q >> 1 : q, j = WPL == 2 ? q & 1 : 0;
-            const uint32_t word = __shfl_sync(0xffffffffu, j == 0 ? wv[0] : wv[1], src);
-            int base = __shfl_sync(0xffffffffu, excl, src);
-            if (j == 1) base += __popc(__shfl_sync(0xffffffffu, wv[0], src));
-            if ((word >> lane) & 1u) {
-                const int b = 32 * q + lane;
-                vals[v0 + base + __popc(word & ((1u << lane) - 1u))] = tx[tile_x_offset(b >> tkl, b & (TK - 1), TK)];
+        V* const tx = x + d * (int64_t)TM * TK;
+        int n = 0;
+        uint32_t mine = 0u;
+        for (int q0 = 0; q0 < BW; q0 += 8) {  // BW is a multiple of 8 (TM, TK >= 16)
+            V h[8];
+            int at[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int b = 32 * (q0 + u) + lane;
+                at[u] = tile_x_offset(b >> tkl, b & (TK - 1), TK);
+                h[u] = tx[at[u]];
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const bool none = TileValue<V>::none(h[u]);
+                const uint32_t word = __ballot_sync(0xffffffffu, !none);
+                if (!none) vals[v0 + n + __popc(word & ((1u << lane) - 1u))] = h[u];
+                else if (sizeof(V) == 2) tx[at[u]] = V(0);
+                if (lane == ((q0 + u) & 31)) mine = word;
+                n += __popc(word);
+            }
+            if (((q0 + 8) & 31) == 0 || q0 + 8 == BW) {  // 32 words, or the last ones
+                const int q = (q0 & ~31) + lane;
+                if (q < BW) bits[d * BW + q] = mine;
             }
         }
+        if (lane < ((8 - (n & 7)) & 7)) vals[v0 + n + lane] = V(0);
     }
 }
 
@@ -894,7 +989,9 @@ __global__ void k_split_tiles(const float* __restrict__ x, int64_t n_eights, int
 {
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n_eights; q += (int64_t)gridDim.x * blockDim.x) {
         const float4 a = __ldg(reinterpret_cast<const float4*>(x) + 2 * q), b = __ldg(reinterpret_cast<const float4*>(x) + 2 * q + 1);
-        const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+        float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = TileValue<float>::none(v[e]) ? 0.f : v[e];
         uint32_t p[3][4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) split3(v[2 * e], v[2 * e + 1], p[0][e], p[1][e], p[2][e]);
@@ -922,6 +1019,52 @@ __global__ void k_window_max(const int32_t* __restrict__ win_ndt, const int32_t*
     if ((threadIdx.x & 31) == 0) {
         atomicMax(reinterpret_cast<unsigned long long*>(out), (unsigned long long)mt);
         atomicMax(reinterpret_cast<unsigned long long*>(out + 1), (unsigned long long)mu);
+    }
+}
+
+// The scans over windows and the maxima in one block, for the plans whose windows a block gets through
+// in a few turns (kScanWindows; more take the device-wide scans): ten launches of 2.5 to 7.5 us each
+// otherwise.
+constexpr int kScanWindows = 8192;
+__global__ void __launch_bounds__(1024) k_window_scans(const int32_t* __restrict__ win_ndt,
+                                                       const int32_t* __restrict__ win_ndv,
+                                                       const int32_t* __restrict__ win_U, int32_t n_win, int32_t TK,
+                                                       int32_t* win_dptr, int64_t* win_vbase, int32_t* dwin,
+                                                       int64_t* totals)
+{
+    __shared__ int64_t sm[1024 / 32 + 1];
+    __shared__ int32_t smax[2];
+    if (threadIdx.x < 2) smax[threadIdx.x] = 0;
+    int64_t carry_t = 0, carry_v = 0;  // (dense windows << 32) + dense tiles; values
+    int32_t mt = 0, mu = 0;
+    for (int w0 = 0; w0 < n_win; w0 += 1024) {
+        const int w = w0 + threadIdx.x;
+        const int32_t nt = w < n_win ? win_ndt[w] : 0;
+        const int64_t nv = w < n_win ? win_ndv[w] : 0;
+        if (w < n_win) {
+            mt = max(mt, nt);
+            mu = max(mu, (win_U[w] + TK - 1) / TK);
+        }
+        int64_t tot_t, tot_v;
+        const int64_t pt = block_excl_scan<int64_t, 1024>(((int64_t)(nt > 0) << 32) + nt, &tot_t, sm) + carry_t;
+        const int64_t pv = block_excl_scan<int64_t, 1024>(nv, &tot_v, sm) + carry_v;
+        if (w < n_win) {
+            win_dptr[w] = (int32_t)(pt & 0xffffffffLL);
+            win_vbase[w] = pv;
+            if (nt > 0) dwin[pt >> 32] = w;
+        }
+        carry_t += tot_t;
+        carry_v += tot_v;
+    }
+    atomicMax(&smax[0], mt);
+    atomicMax(&smax[1], mu);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        totals[1] = carry_t & 0xffffffffLL;
+        totals[2] = carry_v;
+        totals[3] = carry_t >> 32;
+        totals[6] = smax[0];
+        totals[7] = smax[1];
     }
 }
 
@@ -1262,14 +1405,19 @@ ns_status_t window_pass(Plan* P, WindowResult* W, cudaStream_t s)
 
     // ---- W6: scans ----
     NS_CUDA_TRY(cudaMemsetAsync(totals, 0, sizeof(int64_t) * 8, s));
-    NS_TRY(device_scan<int64_t>(I32Load{win_ndt}, PtrStore32{P->win_dptr}, n_win, partial, totals + 1, s));
-    NS_TRY(device_scan<int64_t>(I32Load{win_ndv}, PtrStore64{win_vbase}, n_win, partial, totals + 2, s));
-    NS_TRY(device_scan<int64_t>(DenseWinLoad{win_ndt}, DenseWinStore{P->dwin}, n_win, partial, totals + 3, s));
-    NS_TRY(device_scan<int64_t>(I32Load{res_len}, PtrStore32{P->res_rowptr_own}, m, part2, totals + 4, s));
-    if (n_win > 0) {
-        k_window_max<<<wgrid(n_win), 256, 0, s>>>(win_ndt, win_U, n_win, TK, totals + 6);
+    if (n_win > 0 && n_win <= kScanWindows) {
+        k_window_scans<<<1, 1024, 0, s>>>(win_ndt, win_ndv, win_U, (int32_t)n_win, TK, P->win_dptr, win_vbase, P->dwin, totals);
         NS_LAUNCH_CHECK();
+    } else {
+        NS_TRY(device_scan<int64_t>(I32Load{win_ndt}, PtrStore32{P->win_dptr}, n_win, partial, totals + 1, s));
+        NS_TRY(device_scan<int64_t>(I32Load{win_ndv}, PtrStore64{win_vbase}, n_win, partial, totals + 2, s));
+        NS_TRY(device_scan<int64_t>(DenseWinLoad{win_ndt}, DenseWinStore{P->dwin}, n_win, partial, totals + 3, s));
+        if (n_win > 0) {
+            k_window_max<<<wgrid(n_win), 256, 0, s>>>(win_ndt, win_U, n_win, TK, totals + 6);
+            NS_LAUNCH_CHECK();
+        }
     }
+    NS_TRY(device_scan<int64_t>(I32Load{res_len}, PtrStore32{P->res_rowptr_own}, m, part2, totals + 4, s));
     int64_t ht[8];
     NS_CUDA_TRY(cudaMemcpyAsync(ht, totals, sizeof ht, cudaMemcpyDeviceToHost, s));
     NS_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1290,7 +1438,7 @@ ns_status_t window_pass(Plan* P, WindowResult* W, cudaStream_t s)
     // ---- W7: dense windows, ownership; W8: residual list ----
     NS_CUDA_TRY(cudaMemsetAsync(row_state, 0, (size_t)(m > 0 ? m : 1), s));
     if (n_dwin > 0) {
-        k_dense_windows<<<wgrid(n_dwin), 256, 0, s>>>(P->dwin, n_dwin, win_ndt, win_res, aic_rows, m_aic,
+        k_dense_windows<<<wgrid(n_dwin * 32), 256, 0, s>>>(P->dwin, n_dwin, win_ndt, win_res, aic_rows, m_aic,
                                                       TM, TK, t.absorb_cap, t.cost_tc, t.cost_res,
                                                       P->dwin_absorb, dcost, row_state);
         NS_LAUNCH_CHECK();
@@ -1321,14 +1469,44 @@ ns_status_t window_pass(Plan* P, WindowResult* W, cudaStream_t s)
     P->blocks.push_back(pb.take());
     P->res_col = P->res_col_own;
     P->res_val = P->res_val_own;
-    NS_CUDA_TRY(cudaMemsetAsync(P->dtile_bits, 0, sizeof(uint32_t) * (n_dtiles * BW > 0 ? n_dtiles * BW : 1), s));
-    NS_CUDA_TRY(cudaMemsetAsync(P->dtile_vals, 0, (size_t)(n_dvals > 0 ? n_dvals : 1) * (bf16 ? 2 : 4), s));
-    NS_CUDA_TRY(cudaMemsetAsync(pdense, 0, (size_t)(nnz > 0 ? nnz : 1), s));
+    const bool expand = bf16 || planes;       // the values go through expanded tiles
+    const bool res_done = expand && ident && n_win > 0;  // ... and that pass writes the residual CSR
+    if (!expand) {
+        NS_CUDA_TRY(cudaMemsetAsync(P->dtile_bits, 0, sizeof(uint32_t) * (n_dtiles * BW > 0 ? n_dtiles * BW : 1), s));
+        NS_CUDA_TRY(cudaMemsetAsync(P->dtile_vals, 0, (size_t)(n_dvals > 0 ? n_dvals : 1) * 4, s));
+    }
+    if (!res_done) NS_CUDA_TRY(cudaMemsetAsync(pdense, 0, (size_t)(nnz > 0 ? nnz : 1), s));
     {
         int32_t v32 = (int32_t)n_dvals;
         NS_CUDA_TRY(cudaMemcpyAsync(P->dtile_voff + n_dtiles, &v32, sizeof v32, cudaMemcpyHostToDevice, s));
     }
-    if (n_dtiles > 0) {
+    auto place = [&](auto* tiles) -> ns_status_t {
+        using V = std::remove_pointer_t<decltype(tiles)>;
+        if (n_dtiles > 0) NS_CUDA_TRY(cudaMemsetAsync(tiles, 0xff, sizeof(V) * n_dtiles * TM * TK, s));
+        const int64_t cap = max_ntile * 2 <= kPlaceSmemMax ? max_ntile : 0;
+        PlaceArgs<V> pa2{row_kbase, ident ? nullptr : eidx, epos, ucan, trank, tvoff, win_U, win_ndt, P->win_dptr,
+                         win_vbase, P->vals, m_aic, TM, TK, P->dtile_cols, P->dtile_voff, tiles, pdense, P->colidx,
+                         P->res_rowptr_own, P->res_col_own, P->res_val_own, (int32_t)cap, ilog2(TK)};
+        k_place_tiles<V><<<(unsigned)n_win, kWinThreads, (size_t)cap * 2, s>>>(pa2);
+        NS_LAUNCH_CHECK();
+        if (n_dtiles > 0) {
+            const int64_t blocks = (n_dtiles * 32 + 255) / 256;
+            k_pack_tiles<V><<<(unsigned)(blocks < 65535 * 8 ? blocks : 65535 * 8), 256, 0, s>>>(
+                tiles, P->dtile_voff, n_dtiles, TM, TK, P->dtile_bits, reinterpret_cast<V*>(P->dtile_vals));
+            NS_LAUNCH_CHECK();
+        }
+        return NS_OK;
+    };
+    if (expand && (n_dtiles > 0 || res_done)) {
+        if (bf16) NS_TRY(place(P->dtile_x));
+        else NS_TRY(place(dtile_f));
+        if (!bf16 && n_dtiles > 0) {
+            const int64_t eights = TM * TK / 8;
+            k_split_tiles<<<wgrid(n_dtiles * eights), 256, 0, s>>>(dtile_f, n_dtiles * eights, (int32_t)eights, P->dtile_x);
+            NS_LAUNCH_CHECK();
+        }
+        tf.release(s);
+    } else if (n_dtiles > 0) {
         // shared memory for the largest window, or for as much as fits the limit
         int64_t cap_tiles = max_ntile, cap_words = max_ndt * BW;
         if (cap_tiles * 6 + cap_words * 6 > kEmitSmemMax) {
@@ -1341,31 +1519,12 @@ ns_status_t window_pass(Plan* P, WindowResult* W, cudaStream_t s)
         NS_CUDA_TRY(cudaFuncSetAttribute(k_emit_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kEmitSmemMax + 16));
         EmitArgs ea{row_kbase, eidx, epos, ucan, trank, tvoff, win_U, win_ndt, P->win_dptr, win_vbase,
-                    P->vals, m_aic, TM, TK, bf16 ? 1 : 0, P->dtile_cols, P->dtile_bits, P->dtile_voff,
-                    P->dtile_vals, pdense, (int32_t)cap_words, (int32_t)cap_tiles, ilog2(TK),
-                    bf16 ? P->dtile_x : nullptr, dtile_f};
-        if (bf16) NS_CUDA_TRY(cudaMemsetAsync(P->dtile_x, 0, sizeof(uint16_t) * n_dtiles * TM * TK, s));
-        if (dtile_f) NS_CUDA_TRY(cudaMemsetAsync(dtile_f, 0, sizeof(float) * n_dtiles * TM * TK, s));
+                    P->vals, m_aic, TM, TK, P->dtile_cols, P->dtile_bits, P->dtile_voff,
+                    static_cast<float*>(P->dtile_vals), pdense, (int32_t)cap_words, (int32_t)cap_tiles, ilog2(TK)};
         k_emit_tiles<<<(unsigned)n_win, kWinThreads, dyn, s>>>(ea);
         NS_LAUNCH_CHECK();
-        const int64_t blocks64 = (n_dtiles * 32 + 255) / 256;
-        const unsigned blocks = (unsigned)(blocks64 < 65535 * 8 ? blocks64 : 65535 * 8);
-        if (bf16) {
-            k_pack_tiles<uint16_t><<<blocks, 256, 0, s>>>(P->dtile_bits, P->dtile_voff, P->dtile_x, n_dtiles, TM, TK,
-                                                          reinterpret_cast<uint16_t*>(P->dtile_vals));
-            NS_LAUNCH_CHECK();
-        }
-        if (dtile_f) {
-            k_pack_tiles<float><<<blocks, 256, 0, s>>>(P->dtile_bits, P->dtile_voff, dtile_f, n_dtiles, TM, TK,
-                                                       reinterpret_cast<float*>(P->dtile_vals));
-            NS_LAUNCH_CHECK();
-            const int64_t eights = TM * TK / 8;
-            k_split_tiles<<<wgrid(n_dtiles * eights), 256, 0, s>>>(dtile_f, n_dtiles * eights, (int32_t)eights, P->dtile_x);
-            NS_LAUNCH_CHECK();
-            tf.release(s);
-        }
     }
-    if (m > 0) {
+    if (m > 0 && !res_done) {
         k_residual_scatter<<<wgrid(m * 32), 256, 0, s>>>(P->rowptr, P->colidx, P->vals, pdense,
                                                           P->res_rowptr_own, m, P->res_col_own,
                                                           P->res_val_own);
