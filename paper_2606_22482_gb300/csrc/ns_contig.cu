@@ -27,7 +27,7 @@
 //
 // Cooperative form (plan_coop): when a plan has so few chunks that most warps would get none, the
 // four warps of a CTA share one chunk (4 EPS streams) and the straddling rows meet in shared memory.
-// 4096 rows of 16, K 32: 25.5 -> 13.5 us per call.
+// 4096 rows of 16, K 32: 25.5 -> 13.5 us per call (9.2 since launches report their status themselves).
 #include "ns_internal.cuh"
 #include "ns_mem.cuh"
 

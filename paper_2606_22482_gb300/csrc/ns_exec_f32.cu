@@ -22,7 +22,7 @@
 // issues the MMAs.  The sums then meet the rows' absorbed residual in a shared TM x K tile and the
 // rows are delivered as in the other items.
 //
-// What bounds it (attention mask 32768, TM 64, TK 32, K 128: 834 -> 135 us a launch against the
+// What bounds it (attention mask 32768, TM 64, TK 32, K 128: 834 -> 131 us an execute against the
 // mma.sync item with a three-term TF32 split; error against 64 bits 2.7e-7 -> 1.3e-7): 512 windows
 // on 152 SMs are 3.4 rounds of about 33 us; a tile takes about 0.8 us, its eight small MMAs and the
 // producers' splits about half of that each way, and a window's delivery adds 4 us.  Traffic (240 MB

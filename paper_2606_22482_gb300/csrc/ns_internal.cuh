@@ -180,7 +180,7 @@ struct Plan {
     uint32_t* dtile_bits = nullptr;
     int32_t* dtile_voff = nullptr;
     void* dtile_vals = nullptr;
-    uint16_t* dtile_x = nullptr;  // dense tiles expanded: one plane (BF16) or three (FP32); see k_emit_tiles
+    uint16_t* dtile_x = nullptr;  // dense tiles expanded: one plane (BF16) or three (FP32); see k_place_tiles
     const int32_t* res_rowptr = nullptr;  // aliases rowptr when nothing is dense
     const int32_t* res_col = nullptr;
     const float* res_val = nullptr;

@@ -50,8 +50,10 @@ constexpr size_t count_table_bytes(int64_t n) { return count_words_bytes(n) + (s
 // (2 bytes a word) and its tiles' dense ranks (2 bytes a tile) in dynamic shared memory sized
 // from the plan's largest window, up to this limit (larger windows use global memory)
 constexpr int kEmitSmemMax = 192 * 1024;
-// tile ranks of a window in shared memory (no opt-in needed)
-constexpr int kPlaceSmemMax = 40 * 1024;
+// placement: tile ranks of a window in shared memory (no opt-in needed); rows and threads of a CTA
+constexpr int kPlaceSmemMax = 16 * 1024;
+constexpr int kPlaceRows = 16;
+constexpr int kPlaceThreads = 256;
 
 // ---------------------------------------------------------------------------------------------
 // W1: kept rows
@@ -825,16 +827,21 @@ __global__ void __launch_bounds__(kWinThreads, 4) k_emit_tiles(EmitArgs a)
 }
 
 // W9a: plans that keep expanded tiles (BF16, and FP32 up to kF32TcMaxK columns): each value goes
-// straight to its place in its window's expanded tiles (filled with kNoValue beforehand), one warp
-// per row.  Where the windows hold all of A in CSR order (`ident`), the same pass writes the residual
-// CSR: the row's other elements in order.  Assembling the bitmaps here as well (a segmented OR over
-// the warp and a shared atomic per run), marking dense elements in a byte array and leaving the
-// residual to a pass of its own took 326 + 49 us on the attention mask (32 768 rows, TM 64, TK 32);
-// this takes 291, and planning with one execute 1120 -> 955 us.
+// straight to its place in its window's expanded tiles (filled with the mark of TileValue beforehand), one
+// warp per row.  Where the windows hold all of A in CSR order (IDENT), the same pass writes the residual
+// CSR: the row's other elements in order.  Memory-latency bound; attention mask (32 768 rows, 41 M
+// nonzeros, TM 64, TK 32), this pass:
+//   326 + 49 us  bitmaps assembled here as well (a segmented OR over the warp and a shared atomic per run),
+//                dense elements marked in a byte array for a residual pass of its own
+//   291          bitmaps left to k_pack_tiles, residual written here
+//   240          column ids read with the rest of an element, kept or not (each group of 32 with a kept
+//                one in it waited for memory again), 16 rows a CTA instead of a window
+//   129          the next four elements a lane on their way meanwhile, 32-bit offsets in a row
+// Rows assembled in shared memory and written as whole lines took 646.
 template <class V>
 struct PlaceArgs {
     const int64_t* row_kbase;
-    const int32_t* eidx;  // CSR position of each window element; NULL (ident): element e is position e
+    const int32_t* eidx;  // CSR position of each window element (not IDENT: there element e is position e)
     const int32_t* epos;
     const int32_t* ucan;
     const int32_t* trank;
@@ -873,21 +880,23 @@ struct TileValue<float> {
     static __device__ __forceinline__ bool none(float v) { return __float_as_uint(v) == 0xffffffffu; }
 };
 
-template <class V>
-__global__ void __launch_bounds__(kWinThreads, 3) k_place_tiles(PlaceArgs<V> a)
+template <class V, bool IDENT>
+__global__ void __launch_bounds__(kPlaceThreads, 5) k_place_tiles(PlaceArgs<V> a)
 {
-    __shared__ int64_t rb0[kMaxTM + 1];
+    __shared__ int64_t rb0[kPlaceRows + 1];
     extern __shared__ int16_t place_rank[];
     const int tkl = a.tk_log, TM = a.TM, TK = a.TK;
-    const int w = blockIdx.x;
-    const bool ident = a.eidx == nullptr;
+    const int parts = TM / kPlaceRows;  // CTAs of a window
+    const int w = blockIdx.x / parts, rlo = (blockIdx.x % parts) * kPlaceRows;
     const int32_t ndt = a.win_ndt[w];
-    if (ndt == 0 && !ident) return;
+    if (ndt == 0 && !IDENT) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int64_t r0 = (int64_t)w * TM;
-    const int nrows = (int)(a.m_aic - r0 < TM ? a.m_aic - r0 : TM);
+    const int nwin = (int)(a.m_aic - r0 < TM ? a.m_aic - r0 : TM);
+    if (rlo >= nwin) return;  // (the window's first CTA always has rows)
+    const int nrows = nwin - rlo < kPlaceRows ? nwin - rlo : kPlaceRows;
     const int64_t wbase = a.row_kbase[r0];
-    for (int q = threadIdx.x; q <= nrows; q += blockDim.x) rb0[q] = a.row_kbase[r0 + q] - wbase;
+    for (int q = threadIdx.x; q <= nrows; q += blockDim.x) rb0[q] = a.row_kbase[r0 + rlo + q] - wbase;
     const int64_t U = a.win_U[w];
     const int64_t ntile = (U + TK - 1) / TK;
     const int32_t dbase = a.win_dptr[w];
@@ -895,49 +904,68 @@ __global__ void __launch_bounds__(kWinThreads, 3) k_place_tiles(PlaceArgs<V> a)
     for (int64_t t = threadIdx.x; t < ntile; t += blockDim.x) {
         const int32_t k = a.trank[wbase + t];
         if (in_smem) place_rank[t] = (int16_t)k;
-        if (k >= 0) a.dtile_voff[dbase + k] = (int32_t)(a.win_vbase[w] + a.tvoff[wbase + t]);
+        if (k >= 0 && rlo == 0) a.dtile_voff[dbase + k] = (int32_t)(a.win_vbase[w] + a.tvoff[wbase + t]);
     }
     // columns of the dense tiles: one thread per (tile, column), reads of ucan coalesced
-    for (int64_t q = threadIdx.x; q < ntile * TK; q += blockDim.x) {
+    for (int64_t q = rlo / kPlaceRows * blockDim.x + threadIdx.x; q < ntile * TK; q += ((nwin + kPlaceRows - 1) / kPlaceRows) * blockDim.x) {
         const int32_t k = a.trank[wbase + (q >> tkl)];
         if (k >= 0) a.dtile_cols[(int64_t)(dbase + k) * TK + (q & (TK - 1))] = q < U ? a.ucan[wbase + q] : -1;
     }
     __syncthreads();
     V* const tiles = a.tiles + (int64_t)dbase * TM * TK;
+    const int32_t* const trank = a.trank + wbase;
+    const int tlog = tkl + 31 - __clz(TM);  // values of a tile
     for (int r = warp; r < nrows; r += nwarps) {
-        const int64_t rend = rb0[r + 1];
-        V* const trow = tiles + tile_x_offset(r, 0, TK);
-        int64_t out = ident ? a.res_rowptr[r0 + r] : 0;
-        for (int64_t eb = rb0[r]; eb < rend; eb += 128) {  // four elements per lane in flight
-            int32_t pv[4], iv[4];
-            float vv[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int64_t e = eb + 32 * u + lane;
-                pv[u] = e < rend ? a.epos[wbase + e] : -1;
-                iv[u] = e < rend ? (ident ? (int32_t)(wbase + e) : a.eidx[wbase + e]) : 0;
-                vv[u] = e < rend ? __ldg(a.vals + iv[u]) : 0.f;
+        const int64_t e0 = wbase + rb0[r];
+        const int n = (int)(rb0[r + 1] - rb0[r]);
+        const int32_t* const epos = a.epos + e0;
+        const int32_t* const ids = (IDENT ? a.colidx : a.eidx) + e0;  // column ids, or CSR positions
+        V* const trow = tiles + tile_x_offset(rlo + r, 0, TK);
+        int32_t out = IDENT ? a.res_rowptr[r0 + rlo + r] : 0;
+        // four elements per lane at a time, the next four on their way
+        int32_t pv[4], iv[4];
+        float vv[4];
+        auto load = [&](int e, int32_t& pos, int32_t& id, float& v) {
+            pos = -1, id = 0, v = 0.f;
+            if (e < n) {
+                pos = __ldg(epos + e);
+                id = __ldg(ids + e);
+                if (IDENT) v = __ldg(a.vals + e0 + e);
             }
+        };
+#pragma unroll
+        for (int u = 0; u < 4; ++u) load(32 * u + lane, pv[u], iv[u], vv[u]);
+        for (int eb = 0; eb < n; eb += 128) {
+            int32_t pn[4], in[4];
+            float vn[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) load(eb + 128 + 32 * u + lane, pn[u], in[u], vn[u]);
+            if (!IDENT)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) vv[u] = pv[u] >= 0 ? __ldg(a.vals + iv[u]) : 0.f;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int32_t pos = pv[u];
                 int32_t k = -1;
-                if (pos >= 0) k = in_smem ? (int32_t)place_rank[pos >> tkl] : a.trank[wbase + (pos >> tkl)];
+                if (pos >= 0) k = in_smem ? (int32_t)place_rank[pos >> tkl] : __ldg(trank + (pos >> tkl));
                 if (k >= 0) {
                     const int c = pos & (TK - 1);
-                    trow[(int64_t)k * TM * TK + (c >> 3) * 64 + (c & 7)] = TileValue<V>::of(vv[u]);
-                    if (!ident) a.pdense[iv[u]] = 1;
+                    trow[((int64_t)k << tlog) + ((c & ~7) << 3) + (c & 7)] = TileValue<V>::of(vv[u]);
+                    if (!IDENT) a.pdense[iv[u]] = 1;
                 }
-                if (ident) {
+                if (IDENT) {
                     const bool keep = pos >= 0 && k < 0;
                     const unsigned bal = __ballot_sync(0xffffffffu, keep);
                     if (keep) {
-                        const int64_t o = out + __popc(bal & ((1u << lane) - 1u));
-                        a.res_col[o] = __ldg(a.colidx + iv[u]);
+                        const int32_t o = out + __popc(bal & ((1u << lane) - 1u));
+                        a.res_col[o] = iv[u];
                         a.res_val[o] = vv[u];
                     }
                     out += __popc(bal);
                 }
+                pv[u] = pn[u];
+                iv[u] = in[u];
+                vv[u] = vn[u];
             }
         }
     }
@@ -1492,7 +1520,8 @@ ns_status_t window_pass(Plan* P, WindowResult* W, cudaStream_t s)
         PlaceArgs<V> pa2{row_kbase, ident ? nullptr : eidx, epos, ucan, trank, tvoff, win_U, win_ndt, P->win_dptr,
                          win_vbase, P->vals, m_aic, TM, TK, P->dtile_cols, P->dtile_voff, tiles, pdense, P->colidx,
                          P->res_rowptr_own, P->res_col_own, P->res_val_own, (int32_t)cap, ilog2(TK)};
-        k_place_tiles<V><<<(unsigned)n_win, kWinThreads, (size_t)cap * 2, s>>>(pa2);
+        auto* const kern = ident ? k_place_tiles<V, true> : k_place_tiles<V, false>;
+        kern<<<(unsigned)(n_win * (TM / kPlaceRows)), kPlaceThreads, (size_t)cap * 2, s>>>(pa2);
         NS_LAUNCH_CHECK();
         if (n_dtiles > 0) {
             const int64_t blocks = (n_dtiles * 32 + 255) / 256;
