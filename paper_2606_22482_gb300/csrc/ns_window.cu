@@ -38,12 +38,13 @@ constexpr int kDenseCols = 49152;
 // and, for windows of up to kCanonSmem distinct columns, each column's canonical position (16 bits).
 // The positions take the counters' place, which are not read after the columns are listed: 40 instead
 // of 72 KB for 32 768 columns, so four CTAs fit an SM instead of two and the attention mask's 512
-// windows are one wave instead of two (212 -> 189 us; plan and execute 955 -> 920).
+// windows are one wave instead of two (212 -> 189 us; 171 with 32-bit offsets in the element passes and
+// a column's bits and index in one load).
 constexpr int kCanonSmem = 16384;
 __host__ __device__ constexpr size_t count_words_bytes(int64_t n)
 {
     const size_t counters = (size_t)4 * ((n + 3) / 4), canon = (size_t)2 * (n < kCanonSmem ? n : kCanonSmem);
-    return ((counters > canon ? counters : canon) + 3) & ~(size_t)3;
+    return ((counters > canon ? counters : canon) + 7) & ~(size_t)7;
 }
 constexpr size_t count_table_bytes(int64_t n) { return count_words_bytes(n) + (size_t)8 * ((n + 31) / 32); }
 // emission assembles a window's dense-tile bitmaps (4 bytes a word), their per-tile prefix counts
@@ -284,26 +285,23 @@ __global__ void __launch_bounds__(kWinThreads, 4) k_window_compact(WinArgs a)
     // ---- unique columns of the window in ascending order, with their counts ----
     // Dynamic shared memory: the column counters and positions of the counting path, or (the
     // other path) the two key buffers of an in-shared-memory sort; a CTA takes one of the two.
-    extern __shared__ uint32_t dyn_cols[];
+    extern __shared__ __align__(16) uint32_t dyn_cols[];
     const bool count_cols = a.count_cols && N > kWinSmemKeys;  // window-uniform
     const int nwords = (a.n + 3) >> 2;
     // after the counters: a presence bit per column and, per 32 columns, the ascending index of
     // the first present one; a column's ascending index is then one lookup and a popcount
-    const int ngroups = (a.n + 31) >> 5;
-    uint32_t* const cbits = dyn_cols + count_words_bytes(a.n) / 4;
-    int32_t* const gpre = reinterpret_cast<int32_t*>(cbits + ngroups);
+    uint2* const cidx = reinterpret_cast<uint2*>(dyn_cols + count_words_bytes(a.n) / 4);  // (bits, index)
     uint16_t* const scan = reinterpret_cast<uint16_t*>(dyn_cols);  // canonical position by ascending index
     if (count_cols) {
         // byte counters, four per word (a count is at most TM <= 64)
         for (int q = threadIdx.x; q < nwords; q += blockDim.x) dyn_cols[q] = 0u;
         __syncthreads();
-        for (int64_t e0 = threadIdx.x; e0 < N; e0 += 8 * blockDim.x) {
+        const int n_el = (int)N;  // (a window holds fewer than 2^31 elements)
+        const int32_t* const keys = a.ekey + wbase;
+        for (int e0 = threadIdx.x; e0 < n_el; e0 += 8 * kWinThreads) {
             int32_t cv[8];  // eight column ids per thread in flight
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int64_t e = e0 + (int64_t)u * blockDim.x;
-                cv[u] = e < N ? a.ekey[wbase + e] : -1;
-            }
+            for (int u = 0; u < 8; ++u) cv[u] = n_el - e0 > u * kWinThreads ? __ldg(keys + e0 + u * kWinThreads) : -1;
 #pragma unroll
             for (int u = 0; u < 8; ++u)
                 if (cv[u] >= 0) atomicAdd(&dyn_cols[cv[u] >> 2], 1u << (8 * (cv[u] & 3)));
@@ -351,8 +349,7 @@ __global__ void __launch_bounds__(kWinThreads, 4) k_window_compact(WinArgs a)
                 bw |= __shfl_xor_sync(0xffffffffu, bw, 2);
                 bw |= __shfl_xor_sync(0xffffffffu, bw, 4);
                 if ((lane & 7) == 0 && q < whi) {
-                    cbits[q >> 3] = bw;
-                    gpre[q >> 3] = (int32_t)pre;
+                    cidx[q >> 3] = make_uint2(bw, (uint32_t)pre);
                 }
 #pragma unroll
                 for (int b = 0; b < 4; ++b) {
@@ -500,22 +497,22 @@ __global__ void __launch_bounds__(kWinThreads, 4) k_window_compact(WinArgs a)
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
         for (int r = warp; r < nrows; r += nwarps) {
             int cnt = 0;
-            const int64_t rend = rb0[r + 1];
-            for (int64_t eb = rb0[r]; eb < rend; eb += 128) {  // four column ids per lane in flight
+            const int len = (int)(rb0[r + 1] - rb0[r]);
+            const int32_t* const keys = a.ekey + wbase + rb0[r];
+            int32_t* const rpos = epos + rb0[r];
+            for (int eb = lane; eb - lane < len; eb += 128) {  // four column ids per lane in flight
                 int32_t cv[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int64_t e = eb + 32 * u + lane;
-                    cv[u] = e < rend ? a.ekey[wbase + e] : -1;
-                }
+                for (int u = 0; u < 4; ++u) cv[u] = eb + 32 * u < len ? __ldg(keys + eb + 32 * u) : -1;
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     bool dense = false;
                     if (cv[u] >= 0) {
                         const int32_t c = cv[u];
-                        const int32_t ai = gpre[c >> 5] + __popc(cbits[c >> 5] & ((1u << (c & 31)) - 1u));
+                        const uint2 ci = cidx[c >> 5];
+                        const int32_t ai = (int32_t)ci.y + __popc(ci.x & ((1u << (c & 31)) - 1u));
                         const int32_t pos = U <= kCanonSmem ? (int32_t)scan[ai] : upos[ai];
-                        epos[eb + 32 * u + lane] = pos;
+                        rpos[eb + 32 * u] = pos;
                         const int t = pos >> (TK == 32 ? 5 : 4);  // TK is 16 or 32
                         dense = (tdense[t >> 5] >> (t & 31)) & 1u;
                     }
@@ -527,15 +524,11 @@ __global__ void __launch_bounds__(kWinThreads, 4) k_window_compact(WinArgs a)
     }
     for (int64_t e = count_cols ? N : threadIdx.x; e < N; e += blockDim.x) {
         const int32_t col = a.ekey[wbase + e];
-        int64_t lo = 0, hi = U;  // ascending index of col: the counters' table, or a lower bound in uasc
-        if (count_cols) {
-            lo = gpre[col >> 5] + __popc(cbits[col >> 5] & ((1u << (col & 31)) - 1u));
-        } else {
-            while (lo < hi) {
-                int64_t mid = (lo + hi) >> 1;
-                if (uasc[mid] < col) lo = mid + 1;
-                else hi = mid;
-            }
+        int64_t lo = 0, hi = U;  // a lower bound in uasc
+        while (lo < hi) {
+            int64_t mid = (lo + hi) >> 1;
+            if (uasc[mid] < col) lo = mid + 1;
+            else hi = mid;
         }
         const int32_t pos = upos[lo];
         epos[e] = pos;
