@@ -192,7 +192,7 @@ static ns_status_t check_K(int32_t K)
 }
 
 ns_status_t plan_create(const ns_csr_t* A, int32_t K, ns_dtype_t b_dtype, const ns_tune_t* tune,
-                        cudaStream_t st, Plan** out)
+                        cudaStream_t st, Plan** out, int64_t plane_cap)
 {
     *out = nullptr;
     NS_TRY(check_csr_args(A));
@@ -215,6 +215,7 @@ ns_status_t plan_create(const ns_csr_t* A, int32_t K, ns_dtype_t b_dtype, const 
     }
     cudaGetDevice(&P->device);
     P->last_stream = st;
+    P->plane_cap = plane_cap;
     ns_status_t r = plan_build(P, A, K, b_dtype, &t, st);
     if (r != NS_OK) {
         cudaStreamSynchronize(st);

@@ -28,6 +28,7 @@ struct Batch {
     struct Group {              // graphs sharing K (one persistent launch each)
         int K = 0;
         bool dense = false;
+        bool planes = true;   // FP32: every plan with dense tiles keeps their planes
         bool contig = false;  // every plan of the group has a contiguous residual stream
         ContigMode mode;      // form of the captured launch when contig
         std::vector<int> graphs;
@@ -134,6 +135,7 @@ ns_status_t ns_batch_plan(const ns_csr_t* As, int32_t count, const int32_t* Ks, 
         for (int gi = 0; gi < (int)G.graphs.size(); ++gi) {
             Plan* P = Bt->plans[G.graphs[gi]];
             G.dense = G.dense || P->st.n_dwin > 0;
+            G.planes = G.planes && (P->st.n_dwin == 0 || plan_planes(P));
             G.contig = (gi == 0 || G.contig) && plan_contig(P);
             int64_t n = P->st.n_items;
             std::vector<int64_t> cost(n);
@@ -242,7 +244,8 @@ ns_status_t ns_batch_execute(ns_batch_t b, const void* const* Bs, float* const* 
         for (auto& G : Bt->groups) {  // occupancy queries and attributes outside the capture
             const bool bf16 = Bt->dtype == NS_BF16;
             if (G.contig) NS_TRY(contig_prepare(G.n_items, G.K, bf16, G.mode, &G.grid));
-            else NS_TRY(exec_prepare(G.n_items, G.K, G.TM, G.TK, bf16, Bt->hint, G.dense, &G.grid, G.W));
+            else NS_TRY(exec_prepare(G.n_items, G.K, G.TM, G.TK, bf16, Bt->hint, G.dense, G.planes, &G.grid,
+                                     G.W));
         }
         // the caller's stream may be the legacy default stream, which cannot be captured: record
         // the launches on a private stream once; the graph then replays on the caller's stream
@@ -255,7 +258,7 @@ ns_status_t ns_batch_execute(ns_batch_t b, const void* const* Bs, float* const* 
                                   G.mode, &G.grid, Bt->cap_stream);
             else
                 r = exec_launch(G.descs_dev, G.queue, G.queue_desc, G.n_items, G.ctrl, G.K, G.TM, G.TK,
-                                Bt->dtype == NS_BF16, Bt->hint, G.dense, &G.grid, Bt->cap_stream, nullptr, G.W);
+                                Bt->dtype == NS_BF16, Bt->hint, G.dense, G.planes, &G.grid, Bt->cap_stream, nullptr, G.W);
             if (r != NS_OK) break;
         }
         cudaGraph_t graph = nullptr;

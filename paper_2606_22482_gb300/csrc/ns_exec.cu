@@ -167,14 +167,12 @@ template <bool BF16, bool HINT, bool DENSE>
 static ExecKernel pick_kernel(int K)
 {
     const int nv = K / 4;
-    if constexpr (!DENSE || BF16) {  // (FP32 plans with dense tiles and K <= 256: ns_exec_f32.cu)
-        if (nv <= 2) return k_exec<2, 1, BF16, HINT, DENSE>;
-        if (nv <= 4) return k_exec<4, 1, BF16, HINT, DENSE>;
-        if (nv <= 8) return k_exec<8, 1, BF16, HINT, DENSE>;
-        if (nv <= 16) return k_exec<16, 1, BF16, HINT, DENSE>;
-        if (nv <= 32) return k_exec<32, 1, BF16, HINT, DENSE>;
-        if (nv <= 64) return k_exec<32, 2, BF16, HINT, DENSE>;
-    }
+    if (nv <= 2) return k_exec<2, 1, BF16, HINT, DENSE>;
+    if (nv <= 4) return k_exec<4, 1, BF16, HINT, DENSE>;
+    if (nv <= 8) return k_exec<8, 1, BF16, HINT, DENSE>;
+    if (nv <= 16) return k_exec<16, 1, BF16, HINT, DENSE>;
+    if (nv <= 32) return k_exec<32, 1, BF16, HINT, DENSE>;
+    if (nv <= 64) return k_exec<32, 2, BF16, HINT, DENSE>;
     if (nv <= 128) return k_exec<32, 4, BF16, HINT, DENSE>;
     return k_exec<32, 8, BF16, HINT, DENSE>;
 }
@@ -222,9 +220,9 @@ static size_t exec_smem_bytes(int K, int TM, int TK, bool bf16, bool dense, int 
 // Kernel attributes and the persistent grid (resident CTAs on every SM, at most n_items).
 // Must run outside stream capture.
 ns_status_t exec_prepare(int64_t n_items, int K, int TM, int TK, bool bf16, bool hint, bool dense,
-                         int* grid_out, int W)
+                         bool planes, int* grid_out, int W)
 {
-    if (dense && !bf16 && K <= kF32TcMaxK) return f32_prepare(n_items, K, TM, TK, hint, W, grid_out);
+    if (dense && planes && K <= kF32TcMaxK) return f32_prepare(n_items, K, TM, TK, hint, W, grid_out);
     ExecKernel kern = select_kernel(K, bf16, hint, dense);
     const size_t smem = exec_smem_bytes(K, TM, TK, bf16, dense, W);
     if (smem > 48 * 1024) NS_TRY(dense_prepare(reinterpret_cast<const void*>(kern), smem));
@@ -256,18 +254,19 @@ ns_status_t exec_prepare(int64_t n_items, int K, int TM, int TK, bool bf16, bool
 
 // One persistent launch over `n_items` work items.  queue[t] is an item id of descriptor
 // queue_desc[t] (descriptor 0 when queue_desc is NULL).  All descriptors share K, dtype and L2
-// policy; `dense` selects the kernel with the tensor-core item compiled in.  *grid_cache keeps
+// policy; `dense` selects the kernel with the tensor-core item compiled in, `planes` (every dense
+// plan of an FP32 launch keeps its tiles' planes) the tcgen05 one up to kF32TcMaxK.  *grid_cache keeps
 // the occupancy-derived grid between launches (0 = compute).
 ns_status_t exec_launch(const ExecDesc* descs, const int32_t* queue, const int32_t* queue_desc,
                         int64_t n_items, int32_t* ctrl, int K, int TM, int TK, bool bf16, bool hint,
-                        bool dense, int* grid_cache, cudaStream_t s, const ExecDesc* d0, int W)
+                        bool dense, bool planes, int* grid_cache, cudaStream_t s, const ExecDesc* d0, int W)
 {
-    if (dense && !bf16 && K <= kF32TcMaxK)
+    if (dense && planes && K <= kF32TcMaxK)
         return f32_launch(descs, queue, queue_desc, n_items, ctrl, K, TM, TK, hint, W, grid_cache, s, d0);
     ExecKernel kern = select_kernel(K, bf16, hint, dense);
     const size_t smem = exec_smem_bytes(K, TM, TK, bf16, dense, W);
     int grid = grid_cache ? *grid_cache : 0;
-    if (grid == 0) NS_TRY(exec_prepare(n_items, K, TM, TK, bf16, hint, dense, &grid, W));
+    if (grid == 0) NS_TRY(exec_prepare(n_items, K, TM, TK, bf16, hint, dense, planes, &grid, W));
     if (grid_cache) *grid_cache = grid;
     if (n_items == 0) return NS_OK;
     ExecDesc dv{};
@@ -298,7 +297,7 @@ ns_status_t exec_launch_plan(Plan* P, cudaStream_t s)
     }
     return exec_launch(nullptr, P->queue, nullptr, P->st.n_items, P->ctrl, K, P->tune.TM,
                        P->tune.TK, P->dtype == NS_BF16, P->tune.l2_hints != 0, P->st.n_dwin > 0,
-                       gc, s, &P->desc_host, P->tune.chunk_nnz);
+                       plan_planes(P), gc, s, &P->desc_host, P->tune.chunk_nnz);
 }
 
 }  // namespace ns

@@ -162,6 +162,7 @@ struct Plan {
     ns_plan_stats_t st{};
     ns_tune_t tune{};
     ns_dtype_t dtype = NS_F32;
+    int64_t plane_cap = INT64_MAX;  // bytes the planes of its FP32 tiles may take at most
     int32_t K = 0;
     int device = 0;
 
@@ -251,14 +252,16 @@ ns_status_t plan_check_tune(const ns_tune_t& t);
 void fill_desc(const Plan* P, const void* B, int64_t ldb, float* C, int64_t ldc, ExecDesc* d);
 ns_status_t exec_launch(const ExecDesc* descs, const int32_t* queue, const int32_t* queue_desc,
                         int64_t n_items, int32_t* ctrl, int K, int TM, int TK, bool bf16, bool hint,
-                        bool dense, int* grid_cache, cudaStream_t s, const ExecDesc* d0 = nullptr,
+                        bool dense, bool planes, int* grid_cache, cudaStream_t s, const ExecDesc* d0 = nullptr,
                         int W = 256);
 ns_status_t exec_launch_plan(Plan* P, cudaStream_t s);
 ns_status_t exec_prepare(int64_t n_items, int K, int TM, int TK, bool bf16, bool hint, bool dense,
-                         int* grid_out, int W = 256);
-// FP32 plans with dense tiles, launches of up to kF32TcMaxK columns (ns_exec_f32.cu); such a plan
-// keeps its tiles' planes (dtile_x)
+                         bool planes, int* grid_out, int W = 256);
+// FP32 plans with dense tiles whose planes are kept (dtile_x), launches of up to kF32TcMaxK columns
+// (ns_exec_f32.cu).  A launch of several plans takes this form when all of its dense plans have planes;
+// every plan can take the other one (packed tiles, mma.sync).
 constexpr int kF32TcMaxK = 256;
+inline bool plan_planes(const Plan* P) { return P->dtype == NS_F32 && P->dtile_x != nullptr; }
 ns_status_t f32_prepare(int64_t n_items, int K, int TM, int TK, bool hint, int W, int* grid_out);
 ns_status_t f32_launch(const ExecDesc* descs, const int32_t* queue, const int32_t* queue_desc, int64_t n_items,
                        int32_t* ctrl, int K, int TM, int TK, bool hint, int W, int* grid_cache, cudaStream_t s,
@@ -270,6 +273,7 @@ ns_status_t contig_launch(const ExecDesc* descs, const int32_t* queue, const int
                           const ExecDesc* d0 = nullptr);
 ns_status_t contig_prepare(int64_t n_items, int K, bool bf16, const ContigMode& m, int* grid_out);
 ns_status_t plan_create(const ns_csr_t* A, int32_t K, ns_dtype_t dt, const ns_tune_t* tune,
-                        cudaStream_t s, Plan** out);  // checks + build; on error nothing is kept
+                        cudaStream_t s, Plan** out,   // checks + build; on error nothing is kept
+                        int64_t plane_cap = INT64_MAX);
 
 }  // namespace ns

@@ -209,7 +209,8 @@ static uint64_t plan_key(const ns_tune_t& t, int32_t g, int32_t K, ns_dtype_t dt
     return ((uint64_t)(uint32_t)g << 32) | ((uint64_t)(uint32_t)K << 1) | (uint64_t)(dt == NS_BF16);
 }
 
-// accounted for a plan until the planner has built it: a few bytes per row and per nonzero
+// accounted for a plan until the planner has built it: a few bytes per row and per nonzero (FP32 tiles'
+// planes are not in it: the planner keeps those that fit an eighth of the budget)
 static int64_t est_plan_bytes(const SGraph& g)
 {
     return (int64_t)g.m * 24 + g.nnz * 8 + 4096;
@@ -328,7 +329,8 @@ static void planner_loop(Server* S)
         Plan* P = nullptr;
         std::vector<int32_t> hq;
         std::vector<int8_t> hcls;
-        ns_status_t r = plan_create(&A, sp->K, sp->dt, &S->cfg.tune, S->s_plan, &P);
+        ns_status_t r = plan_create(&A, sp->K, sp->dt, &S->cfg.tune, S->s_plan, &P,
+                                    S->cfg.hbm_budget_bytes / 8);
         if (r == NS_OK) r = host_work_list(P, S->s_plan, &hq, &hcls);
         std::lock_guard<std::mutex> lk(S->mu);
         if (r != NS_OK) {
@@ -511,7 +513,8 @@ static void prepare(Server* S, std::vector<SReq*>& fresh, std::vector<SReq*>& re
 }
 
 // one persistent launch for a group of requests sharing size class, K, dtype and kernel
-static void launch_group(Server* S, std::vector<SReq*>& rs, int cls, int K, bool bf16, bool dense, int TM, int TK)
+static void launch_group(Server* S, std::vector<SReq*>& rs, int cls, int K, bool bf16, bool dense, bool planes, int TM,
+                         int TK)
 {
     struct It {
         int cls;
@@ -594,7 +597,7 @@ static void launch_group(Server* S, std::vector<SReq*>& rs, int cls, int K, bool
     int grid = 0;
     if (cls) {
         const ns_status_t pr = contig ? contig_prepare(ni, K, bf16, mode, &grid)
-                                      : exec_prepare(ni, K, TM, TK, bf16, S->cfg.tune.l2_hints != 0, dense, &grid,
+                                      : exec_prepare(ni, K, TM, TK, bf16, S->cfg.tune.l2_hints != 0, dense, planes, &grid,
                                                      S->cfg.tune.chunk_nnz);
         if (pr != NS_OK) grid = 0;
         grid = grid > 4 ? grid * 3 / 4 : grid;
@@ -604,7 +607,7 @@ static void launch_group(Server* S, std::vector<SReq*>& rs, int cls, int K, bool
     int32_t* const dqd = reinterpret_cast<int32_t*>(base + bD + bQ);
     int32_t* const dctrl = reinterpret_cast<int32_t*>(base + bD + 2 * bQ);
     ns_status_t r = contig ? contig_launch(dd, dq, dqd, ni, dctrl, K, bf16, mode, &grid, es)
-                           : exec_launch(dd, dq, dqd, ni, dctrl, K, TM, TK, bf16, S->cfg.tune.l2_hints != 0, dense,
+                           : exec_launch(dd, dq, dqd, ni, dctrl, K, TM, TK, bf16, S->cfg.tune.l2_hints != 0, dense, planes,
                                          &grid, es, nullptr, S->cfg.tune.chunk_nnz);
     cudaEventCreate(&L.exec_ev);
     cudaEventRecord(L.exec_ev, es);
@@ -722,15 +725,16 @@ static void worker_loop(Server* S)
             std::map<std::tuple<int, int, int, int, int, int, int>, std::vector<SReq*>> groups;
             for (SReq* q : ready) {
                 const Plan* P = q->sp->plan;
-                // kernel form: plans with few chunks take the cooperative form, so they launch apart
-                const int form = plan_contig(P) ? (plan_coop(P) ? 2 : 1) : 0;
+                // kernel form: plans with few chunks take the cooperative form, so they launch apart, and
+                // so do FP32 plans that keep their dense tiles' planes
+                const int form = plan_contig(P) ? (plan_coop(P) ? 2 : 1) : plan_planes(P) ? 3 : 0;
                 groups[{q->cls, q->r.K, (int)q->r.b_dtype, P->st.n_dwin > 0 ? 1 : 0, P->tune.TM, P->tune.TK, form}]
                     .push_back(q);
             }
             for (auto& kv : groups)  // small class first
                 launch_group(S, kv.second, std::get<0>(kv.first), std::get<1>(kv.first),
-                             std::get<2>(kv.first) == NS_BF16, std::get<3>(kv.first) != 0, std::get<4>(kv.first),
-                             std::get<5>(kv.first));
+                             std::get<2>(kv.first) == NS_BF16, std::get<3>(kv.first) != 0, std::get<6>(kv.first) == 3,
+                             std::get<4>(kv.first), std::get<5>(kv.first));
         }
         retire(S);
     }

@@ -644,7 +644,8 @@ struct RlStore {
 };
 
 // ---------------------------------------------------------------------------------------------
-// W9: emit dense tiles (one CTA per window) of plans without expanded tiles (FP32, K > kF32TcMaxK)
+// W9: emit dense tiles (one CTA per window) of plans without expanded tiles (FP32, wider than kF32TcMaxK
+// columns or with planes past their bound)
 // ---------------------------------------------------------------------------------------------
 struct EmitArgs {
     const int64_t* row_kbase;
@@ -821,9 +822,10 @@ __global__ void __launch_bounds__(kWinThreads, 4) k_emit_tiles(EmitArgs a)
 
 // W9a: plans that keep expanded tiles (BF16, and FP32 up to kF32TcMaxK columns): each value goes
 // straight to its place in its window's expanded tiles (filled with the mark of TileValue beforehand), one
-// warp per row.  Where the windows hold all of A in CSR order (IDENT), the same pass writes the residual
-// CSR: the row's other elements in order.  Memory-latency bound; attention mask (32 768 rows, 41 M
-// nonzeros, TM 64, TK 32), this pass:
+// warp per row.  An FP32 tile's values stand at the front of the tile's three planes, which take their
+// place afterwards (k_split_tiles): no second array of tiles.  Where the windows hold all of A in CSR order
+// (IDENT), the same pass writes the residual CSR: the row's other elements in order.  Memory-latency bound;
+// attention mask (32 768 rows, 41 M nonzeros, TM 64, TK 32), this pass:
 //   326 + 49 us  bitmaps assembled here as well (a segmented OR over the warp and a shared atomic per run),
 //                dense elements marked in a byte array for a residual pass of its own
 //   291          bitmaps left to k_pack_tiles, residual written here
@@ -859,18 +861,21 @@ struct PlaceArgs {
 };
 
 // No value of a tile has these bits: the BF16 cast gives NaNs another pattern, and an FP32 NaN of all
-// ones is stored as the NaN next to it.
+// ones is stored as the NaN next to it.  span: how far apart the values are that n places separate, in whole
+// tiles (an FP32 tile takes 6 bytes a place).
 template <class V>
 struct TileValue;
 template <>
 struct TileValue<uint16_t> {
     static __device__ __forceinline__ uint16_t of(float v) { return __bfloat16_as_ushort(__float2bfloat16_rn(v)); }
     static __device__ __forceinline__ bool none(uint16_t h) { return h == 0xffffu; }
+    static __device__ __forceinline__ int64_t span(int64_t n) { return n; }
 };
 template <>
 struct TileValue<float> {
     static __device__ __forceinline__ float of(float v) { return none(v) ? __uint_as_float(0xfffffffeu) : v; }
     static __device__ __forceinline__ bool none(float v) { return __float_as_uint(v) == 0xffffffffu; }
+    static __device__ __forceinline__ int64_t span(int64_t n) { return n + n / 2; }
 };
 
 template <class V, bool IDENT>
@@ -905,7 +910,7 @@ __global__ void __launch_bounds__(kPlaceThreads, 5) k_place_tiles(PlaceArgs<V> a
         if (k >= 0) a.dtile_cols[(int64_t)(dbase + k) * TK + (q & (TK - 1))] = q < U ? a.ucan[wbase + q] : -1;
     }
     __syncthreads();
-    V* const tiles = a.tiles + (int64_t)dbase * TM * TK;
+    V* const tiles = a.tiles + TileValue<V>::span((int64_t)dbase * TM * TK);
     const int32_t* const trank = a.trank + wbase;
     const int tlog = tkl + 31 - __clz(TM);  // values of a tile
     for (int r = warp; r < nrows; r += nwarps) {
@@ -943,7 +948,7 @@ __global__ void __launch_bounds__(kPlaceThreads, 5) k_place_tiles(PlaceArgs<V> a
                 if (pos >= 0) k = in_smem ? (int32_t)place_rank[pos >> tkl] : __ldg(trank + (pos >> tkl));
                 if (k >= 0) {
                     const int c = pos & (TK - 1);
-                    trow[((int64_t)k << tlog) + ((c & ~7) << 3) + (c & 7)] = TileValue<V>::of(vv[u]);
+                    trow[TileValue<V>::span((int64_t)k << tlog) + ((c & ~7) << 3) + (c & 7)] = TileValue<V>::of(vv[u]);
                     if (!IDENT) a.pdense[iv[u]] = 1;
                 }
                 if (IDENT) {
@@ -977,7 +982,7 @@ __global__ void k_pack_tiles(V* __restrict__ x, const int32_t* __restrict__ voff
     for (int64_t d = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; d < n_dtiles;
          d += ((int64_t)gridDim.x * blockDim.x) >> 5) {
         const int64_t v0 = __ldg(voff + d);
-        V* const tx = x + d * (int64_t)TM * TK;
+        V* const tx = x + TileValue<V>::span(d * (int64_t)TM * TK);
         int n = 0;
         uint32_t mine = 0u;
         for (int q0 = 0; q0 < BW; q0 += 8) {  // BW is a multiple of 8 (TM, TK >= 16)
@@ -1009,22 +1014,28 @@ __global__ void k_pack_tiles(V* __restrict__ x, const int32_t* __restrict__ voff
 
 // W9c: FP32 plans, the three BF16 planes of every expanded tile (x = x0 + x1 + x2: x0 truncated, so
 // that it never overflows, x1 and x2 rounded to nearest), plane after plane in each tile, all in the
-// layout of tile_x_offset.  A thread splits eight consecutive elements: 32 bytes in, three times 16
-// bytes out, all coalesced.
-__global__ void k_split_tiles(const float* __restrict__ x, int64_t n_eights, int32_t eights, uint16_t* __restrict__ planes)
+// layout of tile_x_offset.  In place: a block reads whole tiles, 8 values a thread, before any of their
+// planes is written (6 bytes a value on 4); 32 bytes in and three times 16 bytes out, all coalesced.
+constexpr int kSplitThreads = 256;  // 8 values each: one tile of 64 x 32, eight of 16 x 16
+__global__ void __launch_bounds__(kSplitThreads) k_split_tiles(uint16_t* tiles, int64_t n_dtiles, int32_t eights)
 {
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n_eights; q += (int64_t)gridDim.x * blockDim.x) {
-        const float4 a = __ldg(reinterpret_cast<const float4*>(x) + 2 * q), b = __ldg(reinterpret_cast<const float4*>(x) + 2 * q + 1);
-        float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = TileValue<float>::none(v[e]) ? 0.f : v[e];
+    const int per = kSplitThreads / eights, e8 = threadIdx.x % eights;
+    for (int64_t d0 = (int64_t)blockIdx.x * per; d0 < n_dtiles; d0 += (int64_t)gridDim.x * per) {
+        const int64_t d = d0 + threadIdx.x / eights;
+        uint4* const tile = reinterpret_cast<uint4*>(tiles) + d * 3 * eights;
         uint32_t p[3][4];
+        if (d < n_dtiles) {
+            const float4 a = reinterpret_cast<const float4*>(tile)[2 * e8], b = reinterpret_cast<const float4*>(tile)[2 * e8 + 1];
+            float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
-        for (int e = 0; e < 4; ++e) split3(v[2 * e], v[2 * e + 1], p[0][e], p[1][e], p[2][e]);
-        const int64_t tile = q / eights;
-        uint4* out = reinterpret_cast<uint4*>(planes) + tile * 3 * eights + (q - tile * eights);
+            for (int e = 0; e < 8; ++e) v[e] = TileValue<float>::none(v[e]) ? 0.f : v[e];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) out[(int64_t)k * eights] = make_uint4(p[k][0], p[k][1], p[k][2], p[k][3]);
+            for (int e = 0; e < 4; ++e) split3(v[2 * e], v[2 * e + 1], p[0][e], p[1][e], p[2][e]);
+        }
+        __syncthreads();  // the block's tiles are in registers
+        if (d < n_dtiles)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) tile[k * eights + e8] = make_uint4(p[k][0], p[k][1], p[k][2], p[k][3]);
     }
 }
 
@@ -1290,6 +1301,15 @@ __global__ void __launch_bounds__(kReorderThreads) k_local_reorder(
     }
 }
 
+// FP32 planes take 6 TM TK bytes a tile whatever its density, packed tiles TM TK / 8 and 4 a value: up to
+// 1 GiB they are kept (sparse tiles too run 1.7 to 9.8 times as fast from planes: RMAT graphs of 2^15 and
+// 2^17 nodes, tau 1, K 8 to 128), larger ones while they are at most 16 times the CSR's bytes.  A full tile
+// of 16 x 16 holds 16 values at least, 12 times their CSR bytes; tiles of 64 x 32 are within the bound
+// from a mean of 4.7 % filled places on.
+constexpr int64_t kPlaneBytes = 1ll << 30;
+constexpr int64_t kPlaneCsrMultiple = 16;
+static int64_t plane_bytes(int64_t n_dtiles, int TM, int TK) { return 6 * n_dtiles * TM * TK; }
+
 ns_status_t window_pass(Plan* P, WindowResult* W, cudaStream_t s)
 {
     const ns_tune_t& t = P->tune;
@@ -1480,19 +1500,23 @@ ns_status_t window_pass(Plan* P, WindowResult* W, cudaStream_t s)
     pb.reserve_bytes(&P->dtile_vals, (size_t)(n_dvals > 0 ? n_dvals : 1) * (bf16 ? 2 : 4));
     pb.reserve(&P->res_col_own, n_res);
     pb.reserve(&P->res_val_own, n_res);
-    // FP32: planes for the launches of up to kF32TcMaxK columns (the whole width, or a column slice)
-    const int32_t K = P->K, TN = t.TN > 0 && t.TN < K ? t.TN : K;
-    const bool planes = !bf16 && (TN <= kF32TcMaxK || (K % TN != 0 && K % TN <= kF32TcMaxK));
-    float* dtile_f = nullptr;
-    Arena tf;  // temporary
-    if (planes && n_dtiles > 0) {
-        tf.reserve(&dtile_f, n_dtiles * TM * TK);
-        NS_TRY(tf.commit(s));
-    }
     if (bf16) pb.reserve(&P->dtile_x, n_dtiles * TM * TK);
-    if (planes) pb.reserve(&P->dtile_x, 3 * n_dtiles * TM * TK);
     NS_TRY(pb.commit(s));
     P->blocks.push_back(pb.take());
+    // FP32: planes for the launches of up to kF32TcMaxK columns (the whole width, or a column slice),
+    // while they fit their bounds and the device; without them the plan runs from its packed tiles
+    const int32_t K = P->K, TN = t.TN > 0 && t.TN < K ? t.TN : K;
+    const int64_t x_bytes = plane_bytes(n_dtiles, TM, TK), csr_bytes = 8 * nnz + 4 * (m + 1);
+    bool planes = !bf16 && (TN <= kF32TcMaxK || (K % TN != 0 && K % TN <= kF32TcMaxK)) && x_bytes <= P->plane_cap &&
+                  (x_bytes <= kPlaneBytes || x_bytes <= kPlaneCsrMultiple * csr_bytes);
+    if (planes && n_dtiles > 0) {
+        Arena px;
+        px.reserve_bytes(reinterpret_cast<void**>(&P->dtile_x), (size_t)x_bytes);
+        const ns_status_t r = px.commit(s);
+        if (r == NS_OK) P->blocks.push_back(px.take());
+        else if (r == NS_ERR_OOM) planes = false;
+        else return r;
+    }
     P->res_col = P->res_col_own;
     P->res_val = P->res_val_own;
     const bool expand = bf16 || planes;       // the values go through expanded tiles
@@ -1508,7 +1532,7 @@ ns_status_t window_pass(Plan* P, WindowResult* W, cudaStream_t s)
     }
     auto place = [&](auto* tiles) -> ns_status_t {
         using V = std::remove_pointer_t<decltype(tiles)>;
-        if (n_dtiles > 0) NS_CUDA_TRY(cudaMemsetAsync(tiles, 0xff, sizeof(V) * n_dtiles * TM * TK, s));
+        if (n_dtiles > 0) NS_CUDA_TRY(cudaMemsetAsync(tiles, 0xff, bf16 ? 2 * n_dtiles * TM * TK : x_bytes, s));
         const int64_t cap = max_ntile * 2 <= kPlaceSmemMax ? max_ntile : 0;
         PlaceArgs<V> pa2{row_kbase, ident ? nullptr : eidx, epos, ucan, trank, tvoff, win_U, win_ndt, P->win_dptr,
                          win_vbase, P->vals, m_aic, TM, TK, P->dtile_cols, P->dtile_voff, tiles, pdense, P->colidx,
@@ -1526,13 +1550,13 @@ ns_status_t window_pass(Plan* P, WindowResult* W, cudaStream_t s)
     };
     if (expand && (n_dtiles > 0 || res_done)) {
         if (bf16) NS_TRY(place(P->dtile_x));
-        else NS_TRY(place(dtile_f));
+        else NS_TRY(place(reinterpret_cast<float*>(P->dtile_x)));
         if (!bf16 && n_dtiles > 0) {
             const int64_t eights = TM * TK / 8;
-            k_split_tiles<<<wgrid(n_dtiles * eights), 256, 0, s>>>(dtile_f, n_dtiles * eights, (int32_t)eights, P->dtile_x);
+            k_split_tiles<<<wgrid(n_dtiles * eights, kSplitThreads), kSplitThreads, 0, s>>>(P->dtile_x, n_dtiles,
+                                                                                            (int32_t)eights);
             NS_LAUNCH_CHECK();
         }
-        tf.release(s);
     } else if (n_dtiles > 0) {
         // shared memory for the largest window, or for as much as fits the limit
         int64_t cap_tiles = max_ntile, cap_words = max_ndt * BW;
