@@ -224,13 +224,13 @@ ns_status_t ns_batch_execute(ns_batch_t b, const void* const* Bs, float* const* 
             NS_CUDA_TRY(cudaStreamSynchronize(st));  // d is a local buffer
         }
     }
-    // the form of each contiguous-stream launch: 32-byte loads need every B of the group aligned
+    // the form of each contiguous-stream launch: FP32's 32-byte loads need every B of the group aligned
     for (auto& G : Bt->groups) {
         ContigMode m;
-        for (int g : G.graphs) m.b32 = m.b32 && (reinterpret_cast<uintptr_t>(Bs[g]) & 31u) == 0;
+        for (int g : G.graphs) m.any = m.any || contig_any(Bs[g], G.K, Bt->dtype == NS_BF16);
         m.coop = G.n_items * kExecWarps <= 8 * (int64_t)num_sms(Bt->plans[G.graphs[0]]->device);
         m.W = G.W;
-        if (Bt->exec && G.contig && m.b32 != G.mode.b32) {  // captured for the other alignment
+        if (Bt->exec && G.contig && m.any != G.mode.any) {  // captured for the other alignment
             NS_CUDA_TRY(cudaStreamSynchronize(Bt->graph_stream));
             cudaGraphExecDestroy(Bt->exec);
             cudaGraphDestroy(Bt->graph);

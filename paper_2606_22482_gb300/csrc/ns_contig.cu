@@ -31,11 +31,17 @@
 #include "ns_internal.cuh"
 #include "ns_mem.cuh"
 
+#include <type_traits>
+
 namespace ns {
 
-constexpr int kFormF32 = 0;    // B rows 32-byte aligned: one 32-byte load per lane
-constexpr int kFormF32x2 = 1;  // B rows 16-byte aligned: two 16-byte loads
-constexpr int kFormBf16 = 2;   // one 16-byte load of 8 BF16
+constexpr int kFormF32 = 0;      // B rows 32-byte aligned: one 32-byte load per lane
+constexpr int kFormF32Any = 1;   // B rows 16-byte aligned, any distance apart: two 16-byte loads
+constexpr int kFormBf16 = 2;     // one 16-byte load of 8 BF16
+constexpr int kFormBf16Any = 3;  // ... of rows any distance apart
+// (the other forms keep the distance in 32 bits of bytes: one multiply an address, and a register less)
+constexpr bool form_bf16(int form) { return form >= kFormBf16; }
+constexpr bool form_any(int form) { return form == kFormF32Any || form == kFormBf16Any; }
 
 typedef unsigned long long u64;
 
@@ -65,14 +71,14 @@ __device__ __forceinline__ u64 add2(u64 a, u64 b)
 }
 
 // the raw form of 8 columns of a gathered row
-template <int FORM>
-struct Gathered {
+struct GatheredF32 {
     u64 v[4];
 };
-template <>
-struct Gathered<kFormBf16> {
+struct GatheredBf16 {
     uint4 v;
 };
+template <int FORM>
+using Gathered = std::conditional_t<form_bf16(FORM), GatheredBf16, GatheredF32>;
 
 // Loads under a predicate that lives inside the instruction: the destination is read-write, so a
 // skipped load leaves the slot as it was, and no select or copy after the load waits for its data.
@@ -83,7 +89,7 @@ __device__ __forceinline__ void gather8(Gathered<FORM>& r, const unsigned char* 
         asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %6, 0;\n\t"
                      "@q ld.global.nc.L1::no_allocate.L2::cache_hint.v4.b64 {%0,%1,%2,%3}, [%4], %5;\n\t}"
                      : "+l"(r.v[0]), "+l"(r.v[1]), "+l"(r.v[2]), "+l"(r.v[3]) : "l"(p), "l"(pol), "r"((int)on));
-    else if constexpr (FORM == kFormF32x2)
+    else if constexpr (FORM == kFormF32Any)
         asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %6, 0;\n\t"
                      "@q ld.global.nc.L1::no_allocate.L2::cache_hint.v2.b64 {%0,%1}, [%4], %5;\n\t"
                      "@q ld.global.nc.L1::no_allocate.L2::cache_hint.v2.b64 {%2,%3}, [%4 + 16], %5;\n\t}"
@@ -107,7 +113,7 @@ template <int FORM>
 __device__ __forceinline__ void accumulate(u64 (&acc)[4], float w, const Gathered<FORM>& r)
 {
     const u64 ww = pack2(w, w);
-    if constexpr (FORM != kFormBf16) {
+    if constexpr (!form_bf16(FORM)) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[q] = fma2(ww, r.v[q], acc[q]);
     } else {
@@ -239,7 +245,7 @@ __device__ __forceinline__ void contig_chunk(const ExecDesc* Dp, int32_t c, int 
 {
     using Sh = ContigShape<G, FORM>;
     constexpr int EPS = Sh::EPS, DEPTH = Sh::DEPTH, BE = Sh::BE, NB = Sh::NB, MASK = 2 * BE - 1;
-    constexpr int ES = FORM == kFormBf16 ? 2 : 4;
+    constexpr int ES = form_bf16(FORM) ? 2 : 4;
     constexpr int lgE = EPS == 1 ? 0 : EPS == 2 ? 1 : EPS == 4 ? 2 : 3;
     const int g = lane / G, li = lane % G;
     const bool coop = lgU != lgE;  // the CTA's four warps share the chunk
@@ -257,7 +263,7 @@ __device__ __forceinline__ void contig_chunk(const ExecDesc* Dp, int32_t c, int 
 
     // ------------------------------- the chunk and its shares -------------------------------
     unsigned char const* Bl;
-    uint32_t ldb_bytes;
+    std::conditional_t<form_any(FORM), uint64_t, uint32_t> ldb_bytes;
     bool act;            // this lane's 8 columns exist
     int S, Smin;         // every share has Smin or S nonzeros
     int cnt;             // this share's nonzeros
@@ -312,7 +318,7 @@ __device__ __forceinline__ void contig_chunk(const ExecDesc* Dp, int32_t c, int 
         const int col0 = slice * sw + 8 * li;
         act = 8 * li < sw && col0 < D.K;
         Bl = reinterpret_cast<const unsigned char*>(D.B) + (int64_t)col0 * ES;
-        ldb_bytes = (uint32_t)(D.ldb * ES);
+        ldb_bytes = (decltype(ldb_bytes))(D.ldb * ES);
         const int p0 = (total * my) >> lgU, p1 = (total * (my + 1)) >> lgU;
         cnt = p1 - p0;
         S = (total + U - 1) >> lgU;
@@ -484,7 +490,7 @@ __device__ __forceinline__ void contig_chunk(const ExecDesc* Dp, int32_t c, int 
 // CTAs per SM: 7 for 16-lane FP32 groups (power-law 0.68 ms; 0.72 ms at 6 and at 5), 5 for the
 // other FP32 widths (512 graphs, K 64: 2.35 ms; 2.39 ms at 7), 6 for BF16 (0.184 ms; 0.203 ms at 5).
 template <int G, int FORM, bool HOT>
-__global__ void __launch_bounds__(kExecThreads, FORM == kFormBf16 ? 6 : (G == 16 ? 7 : 5)) k_exec_contig(
+__global__ void __launch_bounds__(kExecThreads, form_bf16(FORM) ? 6 : (G == 16 ? 7 : 5)) k_exec_contig(
     const ExecDesc* __restrict__ descs, const int32_t* __restrict__ queue,
     const int32_t* __restrict__ queue_desc, int64_t n_items, int32_t* ctrl, int32_t nsl, int32_t coop,
     const __grid_constant__ ExecDesc d0)
@@ -555,8 +561,9 @@ static ContigKernel pick_contig(int K, bool bf16, const ContigMode& m)
 {
     const int nsl = contig_slices(K);
     const int width = ((K + nsl - 1) / nsl + 7) & ~7;
+    if (m.any)  // (the hot map is only a cache hint)
+        return bf16 ? pick_lanes<kFormBf16Any, false>(width) : pick_lanes<kFormF32Any, false>(width);
     if (bf16) return m.hot ? pick_lanes<kFormBf16, true>(width) : pick_lanes<kFormBf16, false>(width);
-    if (!m.b32) return pick_lanes<kFormF32x2, false>(width);  // (the hot map is only a cache hint)
     return m.hot ? pick_lanes<kFormF32, true>(width) : pick_lanes<kFormF32, false>(width);
 }
 

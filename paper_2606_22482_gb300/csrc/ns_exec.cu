@@ -287,13 +287,13 @@ ns_status_t exec_launch_plan(Plan* P, cudaStream_t s)
     }
     if (plan_contig(P)) {
         ContigMode m;
-        m.b32 = ((reinterpret_cast<uintptr_t>(P->desc_host.B) | (uintptr_t)(P->desc_host.ldb * 4)) & 31u) == 0;
+        m.any = contig_any(P->desc_host.B, P->desc_host.ldb, P->dtype == NS_BF16);
         m.hot = P->hot_bits != nullptr;
         m.coop = plan_coop(P);
         m.W = P->tune.chunk_nnz;
-        // (the cached grid is the 32-byte form's; the other form is rare and asks each time)
+        // (the cached grid is the common form's; the other one is rare and asks each time)
         return contig_launch(nullptr, P->queue, nullptr, P->st.n_items, P->ctrl, K, P->dtype == NS_BF16, m,
-                             m.b32 ? gc : nullptr, s, &P->desc_host);
+                             m.any ? nullptr : gc, s, &P->desc_host);
     }
     return exec_launch(nullptr, P->queue, nullptr, P->st.n_items, P->ctrl, K, P->tune.TM,
                        P->tune.TK, P->dtype == NS_BF16, P->tune.l2_hints != 0, P->st.n_dwin > 0,

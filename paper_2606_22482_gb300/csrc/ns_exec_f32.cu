@@ -153,7 +153,7 @@ __device__ bool ts_window_product(const ExecDesc& D, int32_t w, unsigned char* s
         // (the descriptor's fields once: the loop's memory clobbers would read them again each time)
         const int32_t n = D.n, K = D.K;
         int32_t* const status = D.status;
-        const uint32_t ldb_bytes = (uint32_t)(D.ldb * 4);
+        const int64_t ldb_bytes = D.ldb * 4;
         const unsigned char* const Bw = reinterpret_cast<const unsigned char*>(D.B) + 128 * pw + 16 * (lane & 7);
         // this warp's 32 features of a stage: [column][feature]
         float* const raw = reinterpret_cast<float*>(smem + G.off_b + grp * 2 * TK * 512 + pw * TK * 128);
@@ -191,7 +191,7 @@ __device__ bool ts_window_product(const ExecDesc& D, int32_t w, unsigned char* s
                 const int32_t cc = __shfl_sync(0xffffffffu, col, c + (lane >> 3));
                 if (c < TK) {
                     const bool on = in && cc >= 0;
-                    cp_async16<HINT>(dst + c * 32, src + (on ? (size_t)(uint32_t)cc * ldb_bytes : 0), on, pol.last);
+                    cp_async16<HINT>(dst + c * 32, src + (on ? (int64_t)cc * ldb_bytes : 0), on, pol.last);
                 }
             }
             cp_async_commit();

@@ -234,7 +234,7 @@ int num_sms(int device);
 
 // form of a contiguous-stream launch (ns_contig.cu)
 struct ContigMode {
-    bool b32 = true;    // every row of B starts on a 32-byte boundary
+    bool any = false;   // FP32 rows of B off the 32-byte boundaries, or rows 4 GB or more apart (contig_any)
     bool hot = false;   // single plan with a hot-row map (l2_hints = 2)
     bool coop = false;  // the warps of a CTA share a chunk (plan_coop)
     int W = 256;        // chunk_nnz of the launch's plans
@@ -271,6 +271,11 @@ bool plan_coop(const Plan* P);    // ... with so few chunks that the warps of a 
 ns_status_t contig_launch(const ExecDesc* descs, const int32_t* queue, const int32_t* queue_desc, int64_t n_items,
                           int32_t* ctrl, int K, bool bf16, const ContigMode& m, int* grid_cache, cudaStream_t s,
                           const ExecDesc* d0 = nullptr);
+// B takes the forms for any B: `ldb` elements between rows
+inline bool contig_any(const void* B, int64_t ldb, bool bf16)
+{
+    return ldb > (int64_t)UINT32_MAX / (bf16 ? 2 : 4) || (!bf16 && (reinterpret_cast<uintptr_t>(B) & 31u) != 0);
+}
 ns_status_t contig_prepare(int64_t n_items, int K, bool bf16, const ContigMode& m, int* grid_out);
 ns_status_t plan_create(const ns_csr_t* A, int32_t K, ns_dtype_t dt, const ns_tune_t* tune,
                         cudaStream_t s, Plan** out,   // checks + build; on error nothing is kept

@@ -262,7 +262,7 @@ __device__ __forceinline__ void stream_rows(const ExecDesc& D, int32_t c, int la
     const int nv = D.K >> 2;
     constexpr int VB = BF16 ? 8 : 16;  // bytes of one 4-column vector
     const unsigned char* const Bl = reinterpret_cast<const unsigned char*>(D.B) + VB * lane;
-    const uint32_t ldb_bytes = (uint32_t)(D.ldb * (BF16 ? 2 : 4));
+    const uint64_t ldb_bytes = (uint64_t)D.ldb * (BF16 ? 2 : 4);
     float* const Cp = D.C;
     const int64_t ldc = D.ldc;
 
@@ -301,7 +301,7 @@ __device__ __forceinline__ void stream_rows(const ExecDesc& D, int32_t c, int la
         // padding entries point at a real row with value 0: no test needed here.  With the hot
         // map, bit 31 of the column id marks a hot row (set when the chunk was decoded).
         const uint32_t col = HOT ? ((uint32_t)e.x & 0x7fffffffu) : (uint32_t)e.x;
-        const unsigned char* row = Bl + (size_t)col * ldb_bytes;
+        const unsigned char* row = Bl + (uint64_t)col * ldb_bytes;
         uint64_t pl = pol.last;
         if (HOT) pl = e.x < 0 ? pol.last : pol.first;
 #pragma unroll
