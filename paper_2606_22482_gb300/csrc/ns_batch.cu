@@ -37,7 +37,8 @@ struct Batch {
         int32_t* queue_desc = nullptr;
         int32_t* ctrl = nullptr;
         int64_t n_items = 0;
-        int grid = 0;
+        int grid[2] = {0, 0};  // [1]: the contiguous-stream form for any B
+        cudaGraphNode_t node = nullptr;  // its launch in the graph, when contig
         int TM = 16, TK = 16, W = 256;
     };
     std::vector<Plan*> plans;
@@ -64,6 +65,12 @@ struct Batch {
             if (b.ptr) cudaFree(b.ptr);
     }
 };
+
+// the grid of a contiguous-stream launch's form, asked once
+static ns_status_t contig_grid(Batch::Group& G, bool bf16, const ContigMode& m)
+{
+    return G.grid[m.any] ? NS_OK : contig_prepare(G.n_items, G.K, bf16, m, &G.grid[m.any]);
+}
 
 static int cost_class_host(int64_t c)
 {
@@ -230,12 +237,13 @@ ns_status_t ns_batch_execute(ns_batch_t b, const void* const* Bs, float* const* 
         for (int g : G.graphs) m.any = m.any || contig_any(Bs[g], G.K, Bt->dtype == NS_BF16);
         m.coop = G.n_items * kExecWarps <= 8 * (int64_t)num_sms(Bt->plans[G.graphs[0]]->device);
         m.W = G.W;
-        if (Bt->exec && G.contig && m.any != G.mode.any) {  // captured for the other alignment
-            NS_CUDA_TRY(cudaStreamSynchronize(Bt->graph_stream));
-            cudaGraphExecDestroy(Bt->exec);
-            cudaGraphDestroy(Bt->graph);
-            Bt->exec = nullptr;
-            Bt->graph = nullptr;
+        if (Bt->exec && G.node && m.any != G.mode.any) {  // the launch takes its other form from now on
+            cudaKernelNodeParams np{};
+            NS_CUDA_TRY(cudaGraphKernelNodeGetParams(G.node, &np));
+            NS_TRY(contig_grid(G, Bt->dtype == NS_BF16, m));
+            np.func = const_cast<void*>(contig_kernel(G.K, Bt->dtype == NS_BF16, m));
+            np.gridDim = dim3((unsigned)G.grid[m.any]);
+            NS_CUDA_TRY(cudaGraphExecKernelNodeSetParams(Bt->exec, G.node, &np));
         }
         G.mode = m;
     }
@@ -243,8 +251,8 @@ ns_status_t ns_batch_execute(ns_batch_t b, const void* const* Bs, float* const* 
         // capture every group's persistent launch once; later calls replay the graph
         for (auto& G : Bt->groups) {  // occupancy queries and attributes outside the capture
             const bool bf16 = Bt->dtype == NS_BF16;
-            if (G.contig) NS_TRY(contig_prepare(G.n_items, G.K, bf16, G.mode, &G.grid));
-            else NS_TRY(exec_prepare(G.n_items, G.K, G.TM, G.TK, bf16, Bt->hint, G.dense, G.planes, &G.grid,
+            if (G.contig) NS_TRY(contig_grid(G, bf16, G.mode));
+            else NS_TRY(exec_prepare(G.n_items, G.K, G.TM, G.TK, bf16, Bt->hint, G.dense, G.planes, G.grid,
                                      G.W));
         }
         // the caller's stream may be the legacy default stream, which cannot be captured: record
@@ -255,15 +263,31 @@ ns_status_t ns_batch_execute(ns_batch_t b, const void* const* Bs, float* const* 
         for (auto& G : Bt->groups) {
             if (G.contig)
                 r = contig_launch(G.descs_dev, G.queue, G.queue_desc, G.n_items, G.ctrl, G.K, Bt->dtype == NS_BF16,
-                                  G.mode, &G.grid, Bt->cap_stream);
+                                  G.mode, &G.grid[G.mode.any], Bt->cap_stream);
             else
                 r = exec_launch(G.descs_dev, G.queue, G.queue_desc, G.n_items, G.ctrl, G.K, G.TM, G.TK,
-                                Bt->dtype == NS_BF16, Bt->hint, G.dense, G.planes, &G.grid, Bt->cap_stream, nullptr, G.W);
+                                Bt->dtype == NS_BF16, Bt->hint, G.dense, G.planes, G.grid, Bt->cap_stream, nullptr, G.W);
             if (r != NS_OK) break;
+            if (G.contig && G.n_items > 0) {  // the node just recorded is what the stream now waits for
+                const cudaGraphNode_t* last = nullptr;
+                size_t n = 0;
+                cudaStreamCaptureStatus cs;
+                if (cudaStreamGetCaptureInfo(Bt->cap_stream, &cs, nullptr, nullptr, &last, nullptr, &n) != cudaSuccess ||
+                    n != 1) {
+                    set_error("no node for the captured launch");
+                    r = NS_ERR_CUDA;
+                    break;
+                }
+                G.node = last[0];
+            }
         }
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamEndCapture(Bt->cap_stream, &graph);
-        if (r != NS_OK) return r;
+        if (r != NS_OK) {
+            if (e == cudaSuccess) cudaGraphDestroy(graph);
+            (void)cudaGetLastError();
+            return r;
+        }
         if (e != cudaSuccess) {
             set_error("stream capture failed: %s", cudaGetErrorString(e));
             return NS_ERR_CUDA;

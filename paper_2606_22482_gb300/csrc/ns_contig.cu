@@ -567,6 +567,11 @@ static ContigKernel pick_contig(int K, bool bf16, const ContigMode& m)
     return m.hot ? pick_lanes<kFormF32, true>(width) : pick_lanes<kFormF32, false>(width);
 }
 
+const void* contig_kernel(int K, bool bf16, const ContigMode& m)
+{
+    return reinterpret_cast<const void*>(pick_contig(K, bf16, m));
+}
+
 // the persistent grid: resident CTAs on every SM, at most one per unit of work
 ns_status_t contig_prepare(int64_t n_items, int K, bool bf16, const ContigMode& m, int* grid_out)
 {

@@ -280,20 +280,21 @@ ns_status_t exec_launch(const ExecDesc* descs, const int32_t* queue, const int32
 ns_status_t exec_launch_plan(Plan* P, cudaStream_t s)
 {
     const int K = P->desc_host.K;  // the column slice of this launch
-    int* gc = K == P->K ? &P->exec_grid : &P->exec_grid_slice;
-    if (K != P->K && P->exec_grid_slice_K != K) {
-        P->exec_grid_slice = 0;
-        P->exec_grid_slice_K = K;
+    const bool contig = plan_contig(P);
+    const bool any = contig && contig_any(P->desc_host.B, P->desc_host.ldb, P->dtype == NS_BF16);
+    int* gc = K == P->K ? &P->exec_grid[any] : &P->exec_grid_slice[any];
+    if (K != P->K && P->exec_grid_slice_K[any] != K) {
+        P->exec_grid_slice[any] = 0;
+        P->exec_grid_slice_K[any] = K;
     }
-    if (plan_contig(P)) {
+    if (contig) {
         ContigMode m;
-        m.any = contig_any(P->desc_host.B, P->desc_host.ldb, P->dtype == NS_BF16);
+        m.any = any;
         m.hot = P->hot_bits != nullptr;
         m.coop = plan_coop(P);
         m.W = P->tune.chunk_nnz;
-        // (the cached grid is the common form's; the other one is rare and asks each time)
-        return contig_launch(nullptr, P->queue, nullptr, P->st.n_items, P->ctrl, K, P->dtype == NS_BF16, m,
-                             m.any ? nullptr : gc, s, &P->desc_host);
+        return contig_launch(nullptr, P->queue, nullptr, P->st.n_items, P->ctrl, K, P->dtype == NS_BF16, m, gc, s,
+                             &P->desc_host);
     }
     return exec_launch(nullptr, P->queue, nullptr, P->st.n_items, P->ctrl, K, P->tune.TM,
                        P->tune.TK, P->dtype == NS_BF16, P->tune.l2_hints != 0, P->st.n_dwin > 0,

@@ -209,8 +209,8 @@ struct Plan {
     ExecDesc desc_host{};           // the single-plan descriptor (a kernel parameter)
     bool desc_valid = false;
     std::vector<DevBlock> blocks;  // every device allocation the plan owns
-    int exec_grid = 0;
-    int exec_grid_slice = 0, exec_grid_slice_K = 0;  // grid of the column-slice launches
+    // grids of the launches over all columns and of the column slices' ([1]: the forms for any B)
+    int exec_grid[2] = {0, 0}, exec_grid_slice[2] = {0, 0}, exec_grid_slice_K[2] = {0, 0};
     cudaStream_t last_stream = nullptr;  // stream of the last plan/execute call: frees go there
     volatile int32_t* status_host = nullptr;  // mapped host word: the status a finished launch reported
     int32_t* status_map = nullptr;            // its device address
@@ -277,6 +277,7 @@ inline bool contig_any(const void* B, int64_t ldb, bool bf16)
     return ldb > (int64_t)UINT32_MAX / (bf16 ? 2 : 4) || (!bf16 && (reinterpret_cast<uintptr_t>(B) & 31u) != 0);
 }
 ns_status_t contig_prepare(int64_t n_items, int K, bool bf16, const ContigMode& m, int* grid_out);
+const void* contig_kernel(int K, bool bf16, const ContigMode& m);  // (all of them take the same arguments)
 ns_status_t plan_create(const ns_csr_t* A, int32_t K, ns_dtype_t dt, const ns_tune_t* tune,
                         cudaStream_t s, Plan** out,   // checks + build; on error nothing is kept
                         int64_t plane_cap = INT64_MAX);
