@@ -861,7 +861,7 @@ struct PlaceArgs {
 };
 
 // No value of a tile has these bits: the BF16 cast gives NaNs another pattern, and an FP32 NaN of all
-// ones is stored as the NaN next to it.  span: how far apart the values are that n places separate, in whole
+// ones stands there as the NaN next to it (k_pack_tiles tells the two apart).  span: how far apart the values are that n places separate, in whole
 // tiles (an FP32 tile takes 6 bytes a place).
 template <class V>
 struct TileValue;
@@ -969,12 +969,38 @@ __global__ void __launch_bounds__(kPlaceThreads, 5) k_place_tiles(PlaceArgs<V> a
     }
 }
 
+// Where A keeps the value of a place of a dense tile: the row by its window, the column by the tile's list.
+struct TileSource {
+    const int32_t *win_dptr, *win_rows, *dtile_cols, *rowptr, *colidx;
+    const float* vals;
+    int32_t n_win, TM, TK;
+};
+// (out of line and rare: one NaN pattern asks for it)
+__device__ __noinline__ float tile_source(const TileSource& a, int64_t d, int r, int c)
+{
+    int32_t lo = 0, hi = a.n_win;  // the window that holds tile d
+    while (hi - lo > 1) {
+        const int32_t mid = (lo + hi) >> 1;
+        if (__ldg(a.win_dptr + mid) <= d) lo = mid;
+        else hi = mid;
+    }
+    const int32_t i = __ldg(a.win_rows + (int64_t)lo * a.TM + r), col = __ldg(a.dtile_cols + d * a.TK + c);
+    int64_t p = __ldg(a.rowptr + i), e = __ldg(a.rowptr + i + 1);
+    while (e - p > 1) {  // the columns of a row ascend
+        const int64_t mid = (p + e) >> 1;
+        if (__ldg(a.colidx + mid) <= col) p = mid;
+        else e = mid;
+    }
+    return __ldg(a.vals + p);
+}
+
 // W9b: bitmaps and packed values from the expanded tiles, one warp per tile: 32 elements of the tile at
 // a time in bitmap order; a present value goes to its rank.  BF16 tiles are what the execute kernel
 // multiplies, so their absent places become zeros.  Values are padded to a multiple of 8 with zeros.
 template <class V>
 __global__ void k_pack_tiles(V* __restrict__ x, const int32_t* __restrict__ voff, int64_t n_dtiles, int32_t TM,
-                             int32_t TK, uint32_t* __restrict__ bits, V* __restrict__ vals)
+                             int32_t TK, uint32_t* __restrict__ bits, V* __restrict__ vals,
+                             const __grid_constant__ TileSource src)
 {
     const int lane = threadIdx.x & 31;
     const int BW = TM * TK / 32;
@@ -998,6 +1024,11 @@ __global__ void k_pack_tiles(V* __restrict__ x, const int32_t* __restrict__ voff
             for (int u = 0; u < 8; ++u) {
                 const bool none = TileValue<V>::none(h[u]);
                 const uint32_t word = __ballot_sync(0xffffffffu, !none);
+                if constexpr (sizeof(V) == 4)
+                    if (__float_as_uint(h[u]) == 0xfffffffeu) {
+                        const int b = 32 * (q0 + u) + lane;
+                        h[u] = tile_source(src, d, b >> tkl, b & (TK - 1));
+                    }
                 if (!none) vals[v0 + n + __popc(word & ((1u << lane) - 1u))] = h[u];
                 else if (sizeof(V) == 2) tx[at[u]] = V(0);
                 if (lane == ((q0 + u) & 31)) mine = word;
@@ -1543,7 +1574,8 @@ ns_status_t window_pass(Plan* P, WindowResult* W, cudaStream_t s)
         if (n_dtiles > 0) {
             const int64_t blocks = (n_dtiles * 32 + 255) / 256;
             k_pack_tiles<V><<<(unsigned)(blocks < 65535 * 8 ? blocks : 65535 * 8), 256, 0, s>>>(
-                tiles, P->dtile_voff, n_dtiles, TM, TK, P->dtile_bits, reinterpret_cast<V*>(P->dtile_vals));
+                tiles, P->dtile_voff, n_dtiles, TM, TK, P->dtile_bits, reinterpret_cast<V*>(P->dtile_vals),
+                TileSource{P->win_dptr, P->win_rows, P->dtile_cols, P->rowptr, P->colidx, P->vals, (int32_t)n_win, TM, TK});
             NS_LAUNCH_CHECK();
         }
         return NS_OK;
