@@ -915,7 +915,7 @@ __global__ void __launch_bounds__(kPlaceThreads, 5) k_place_tiles(PlaceArgs<V> a
     const int tlog = tkl + 31 - __clz(TM);  // values of a tile
     for (int r = warp; r < nrows; r += nwarps) {
         const int64_t e0 = wbase + rb0[r];
-        const int n = (int)(rb0[r + 1] - rb0[r]);
+        const uint32_t n = (uint32_t)(rb0[r + 1] - rb0[r]);  // (below 2^31: what is read ahead ends below 2^32)
         const int32_t* const epos = a.epos + e0;
         const int32_t* const ids = (IDENT ? a.colidx : a.eidx) + e0;  // column ids, or CSR positions
         V* const trow = tiles + tile_x_offset(rlo + r, 0, TK);
@@ -923,7 +923,7 @@ __global__ void __launch_bounds__(kPlaceThreads, 5) k_place_tiles(PlaceArgs<V> a
         // four elements per lane at a time, the next four on their way
         int32_t pv[4], iv[4];
         float vv[4];
-        auto load = [&](int e, int32_t& pos, int32_t& id, float& v) {
+        auto load = [&](uint32_t e, int32_t& pos, int32_t& id, float& v) {
             pos = -1, id = 0, v = 0.f;
             if (e < n) {
                 pos = __ldg(epos + e);
@@ -933,7 +933,7 @@ __global__ void __launch_bounds__(kPlaceThreads, 5) k_place_tiles(PlaceArgs<V> a
         };
 #pragma unroll
         for (int u = 0; u < 4; ++u) load(32 * u + lane, pv[u], iv[u], vv[u]);
-        for (int eb = 0; eb < n; eb += 128) {
+        for (uint32_t eb = 0; eb < n; eb += 128) {
             int32_t pn[4], in[4];
             float vn[4];
 #pragma unroll
