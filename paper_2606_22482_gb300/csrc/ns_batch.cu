@@ -40,6 +40,7 @@ struct Batch {
         int grid[2] = {0, 0};  // [1]: the contiguous-stream form for any B
         cudaGraphNode_t node = nullptr;  // its launch in the graph, when contig
         int TM = 16, TK = 16, W = 256;
+        int64_t n_rows = 0;  // of all its B
     };
     std::vector<Plan*> plans;
     std::vector<Group> groups;
@@ -141,9 +142,10 @@ ns_status_t ns_batch_plan(const ns_csr_t* As, int32_t count, const int32_t* Ks, 
         std::vector<It> items;
         for (int gi = 0; gi < (int)G.graphs.size(); ++gi) {
             Plan* P = Bt->plans[G.graphs[gi]];
+            G.n_rows += P->st.n;
             G.dense = G.dense || P->st.n_dwin > 0;
             G.planes = G.planes && (P->st.n_dwin == 0 || plan_planes(P));
-            G.contig = (gi == 0 || G.contig) && plan_contig(P);
+            G.contig = (gi == 0 || G.contig) && contig_form(P, G.K);
             int64_t n = P->st.n_items;
             std::vector<int64_t> cost(n);
             std::vector<int32_t> q(n);
@@ -235,8 +237,8 @@ ns_status_t ns_batch_execute(ns_batch_t b, const void* const* Bs, float* const* 
     for (auto& G : Bt->groups) {
         ContigMode m;
         for (int g : G.graphs) m.any = m.any || contig_any(Bs[g], G.K, Bt->dtype == NS_BF16);
-        m.coop = G.n_items * kExecWarps <= 8 * (int64_t)num_sms(Bt->plans[G.graphs[0]]->device);
-        m.W = G.W;
+        m.far = contig_far(G.n_rows, G.K, Bt->dtype == NS_BF16, Bt->plans[G.graphs[0]]->device);
+        m.coop = contig_coop(G.n_items * kExecWarps, Bt->plans[G.graphs[0]]->device);
         if (Bt->exec && G.node && m.any != G.mode.any) {  // the launch takes its other form from now on
             cudaKernelNodeParams np{};
             NS_CUDA_TRY(cudaGraphKernelNodeGetParams(G.node, &np));

@@ -11,12 +11,13 @@
 // and to the starts of chunks (about 10 us each, a chain of dependent loads).
 //
 // Split of the work: a lane owns 8 adjacent columns (32 bytes of FP32 in one 256-bit load, or 16
-// bytes of BF16), so G = K / 8 lanes cover a row and the warp holds EPS = 32 / G lane groups.
+// bytes of BF16; FP32 off the 32-byte boundaries: 4 in each half of the row), so G = K / 8 lanes cover a row and the warp holds EPS = 32 / G lane groups.
 // Each group is a stream of its own: the chunk's nonzeros are divided equally among the groups,
 // each group walks its share in order and stores its own rows, so a row end costs no sum over the
 // warp.  A row that straddles shares is put together at the end of the chunk: every share but the
 // first one of such a row parks its part in shared memory and the row's first share adds the parts
-// in order.  Sums therefore have a fixed order that depends only on the plan and K.  Gathers run
+// in order.  Sums therefore have a fixed order that depends only on the plan and K (a graph of a batch:
+// and on how many chunks the graphs of its width have together, contig_coop).  Gathers run
 // DEPTH steps ahead in a register ring, so a row crosses the L1 data pipe once; products are packed
 // two columns to an instruction (fma.rn.f32x2, the same rounding as two fmaf).
 //
@@ -24,8 +25,13 @@
 // in shared memory at K = 128; lane groups summed by shuffles at every row end below that):
 //   power-law 2^20, K 128 FP32     0.705 -> 0.679 ms      512 graphs, K 64 FP32   2.93 -> 2.40 ms
 //   300007 nodes, K 96 BF16        0.210 -> 0.184 ms      100003 nodes, K 512     0.313 -> 0.222 ms
+// Where that first form of it was slower, and what it takes now (us before it, then, now; RMAT of 16 a row, W 256):
+//   2^20 nodes, K 32 FP32   339  446  338    batches and a ring half as long for 4-lane groups, one more CTA
+//   2^16 nodes, K 128 FP32   62   74   63    5 CTAs an SM without spills while B is within L2
+//   rows of 700 pieces, K 32 BF16  89  188   50    all lane groups add a split row's pieces
+//   2^17 nodes, K 256 FP32, B on a 16-byte boundary  172  269  154    4 columns of a lane in each half of the row
 //
-// Cooperative form (plan_coop): when a plan has so few chunks that most warps would get none, the
+// Cooperative form (contig_coop): when a launch has so few chunks that most warps would get none, the
 // four warps of a CTA share one chunk (4 EPS streams) and the straddling rows meet in shared memory.
 // 4096 rows of 16, K 32: 25.5 -> 13.5 us per call (9.2 since launches report their status themselves).
 #include "ns_internal.cuh"
@@ -82,18 +88,19 @@ using Gathered = std::conditional_t<form_bf16(FORM), GatheredBf16, GatheredF32>;
 
 // Loads under a predicate that lives inside the instruction: the destination is read-write, so a
 // skipped load leaves the slot as it was, and no select or copy after the load waits for its data.
-template <int FORM>
-__device__ __forceinline__ void gather8(Gathered<FORM>& r, const unsigned char* p, uint64_t pol, bool on)
+template <int FORM, int G>
+__device__ __forceinline__ void gather8(Gathered<FORM>& r, const unsigned char* p, uint64_t pol, bool on, bool on1)
 {
     if constexpr (FORM == kFormF32)
         asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %6, 0;\n\t"
                      "@q ld.global.nc.L1::no_allocate.L2::cache_hint.v4.b64 {%0,%1,%2,%3}, [%4], %5;\n\t}"
                      : "+l"(r.v[0]), "+l"(r.v[1]), "+l"(r.v[2]), "+l"(r.v[3]) : "l"(p), "l"(pol), "r"((int)on));
     else if constexpr (FORM == kFormF32Any)
-        asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %6, 0;\n\t"
+        asm volatile("{\n\t.reg .pred q, q1;\n\tsetp.ne.s32 q, %6, 0;\n\tsetp.ne.s32 q1, %7, 0;\n\t"
                      "@q ld.global.nc.L1::no_allocate.L2::cache_hint.v2.b64 {%0,%1}, [%4], %5;\n\t"
-                     "@q ld.global.nc.L1::no_allocate.L2::cache_hint.v2.b64 {%2,%3}, [%4 + 16], %5;\n\t}"
-                     : "+l"(r.v[0]), "+l"(r.v[1]), "+l"(r.v[2]), "+l"(r.v[3]) : "l"(p), "l"(pol), "r"((int)on));
+                     "@q1 ld.global.nc.L1::no_allocate.L2::cache_hint.v2.b64 {%2,%3}, [%4 + %8], %5;\n\t}"
+                     : "+l"(r.v[0]), "+l"(r.v[1]), "+l"(r.v[2]), "+l"(r.v[3])
+                     : "l"(p), "l"(pol), "r"((int)on), "r"((int)on1), "n"(16 * G));
     else
         asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %6, 0;\n\t"
                      "@q ld.global.nc.L1::no_allocate.L2::cache_hint.v4.b32 {%0,%1,%2,%3}, [%4], %5;\n\t}"
@@ -124,19 +131,29 @@ __device__ __forceinline__ void accumulate(u64 (&acc)[4], float w, const Gathere
     }
 }
 
-__device__ __forceinline__ void store8(float* p, const u64 (&a)[4], uint64_t pol)
+// a lane's two times 4 columns, HI apart, where they exist (both or none of 8 in a row)
+template <int HI>
+__device__ __forceinline__ void store8(float* p, bool act, bool act1, const u64 (&a)[4], uint64_t pol)
 {
     const float2 x = unpack2(a[0]), y = unpack2(a[1]), z = unpack2(a[2]), w = unpack2(a[3]);
-    st_c4<true>(p, make_float4(x.x, x.y, y.x, y.y), pol);
-    st_c4<true>(p + 4, make_float4(z.x, z.y, w.x, w.y), pol);
+    if (act) {
+        st_c4<true>(p, make_float4(x.x, x.y, y.x, y.y), pol);
+        if (HI == 4) st_c4<true>(p + 4, make_float4(z.x, z.y, w.x, w.y), pol);
+    }
+    if (HI != 4 && act1) st_c4<true>(p + HI, make_float4(z.x, z.y, w.x, w.y), pol);
 }
 
 // One piece of a row that several chunks share (out of line: at most two per chunk).  The lanes
-// with `mine` set hold the piece, 8 columns from `col` each where `act`; the whole warp calls.
-// The piece that arrives last sums the pieces in order and stores the row.
-__device__ __noinline__ void deliver_piece(const ExecDesc& D, int32_t row, int32_t c, bool mine, bool act, int col,
-                                           u64 a0, u64 a1, u64 a2, u64 a3, int nsl, int slice, uint64_t pol)
+// with `mine` set hold the piece; the whole warp calls, each lane with the columns that its place in
+// a group of G lanes stands for: 4 from `col` where `act` and 4 from col + HI where `act1`.  The piece that
+// arrives last sums the pieces and stores the row: lane group j adds pieces j, j + 32 / G, ... in order,
+// kAhead of them on their way at a time, then the groups' sums are added in order.
+template <int G, int HI>
+__device__ __noinline__ void deliver_piece(const ExecDesc& D, int32_t row, int32_t c, bool mine, bool act, bool act1,
+                                           int col, u64 a0, u64 a1, u64 a2, u64 a3, int nsl, int slice,
+                                           uint64_t pol)
 {
+    constexpr int EPS = 32 / G, kAhead = G < 32 ? 2 : 4;
     const int lane = threadIdx.x & 31;
     const unsigned who = __ballot_sync(0xffffffffu, mine);
     if (who == 0u) return;
@@ -154,11 +171,11 @@ __device__ __noinline__ void deliver_piece(const ExecDesc& D, int32_t row, int32
         if (lane == 0) atomicOr(D.status, kStatusInternal);
         return;
     }
-    if (mine && act) {
+    if (mine) {
         float* p = slot0 + (int64_t)piece * D.K;
         const float2 x = unpack2(a0), y = unpack2(a1), z = unpack2(a2), w = unpack2(a3);
-        __stcg(reinterpret_cast<float4*>(p), make_float4(x.x, x.y, y.x, y.y));
-        __stcg(reinterpret_cast<float4*>(p + 4), make_float4(z.x, z.y, w.x, w.y));
+        if (act) __stcg(reinterpret_cast<float4*>(p), make_float4(x.x, x.y, y.x, y.y));
+        if (act1) __stcg(reinterpret_cast<float4*>(p + HI), make_float4(z.x, z.y, w.x, w.y));
     }
     __threadfence();
     __syncwarp();
@@ -168,20 +185,33 @@ __device__ __noinline__ void deliver_piece(const ExecDesc& D, int32_t row, int32
     old = __shfl_sync(0xffffffffu, old, 0);
     if (old != np - 1) return;  // not the last piece
     __threadfence();
-    if (mine && act) {
-        u64 sum[4] = {0ull, 0ull, 0ull, 0ull};
-#pragma unroll 8
-        for (int q = 0; q < np; ++q) {
-            const float* p = slot0 + (int64_t)q * D.K;
-            const float4 x = __ldcg(reinterpret_cast<const float4*>(p));
-            const float4 y = __ldcg(reinterpret_cast<const float4*>(p + 4));
-            sum[0] = add2(sum[0], pack2(x.x, x.y));
-            sum[1] = add2(sum[1], pack2(x.z, x.w));
-            sum[2] = add2(sum[2], pack2(y.x, y.y));
-            sum[3] = add2(sum[3], pack2(y.z, y.w));
+    u64 sum[4] = {0ull, 0ull, 0ull, 0ull};
+    for (int q0 = lane / G; q0 < np; q0 += kAhead * EPS) {
+        float4 x[kAhead], y[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const float* p = slot0 + (int64_t)(q0 + u * EPS) * D.K;
+            const bool in = q0 + u * EPS < np;
+            x[u] = y[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (in && act) x[u] = __ldcg(reinterpret_cast<const float4*>(p));
+            if (in && act1) y[u] = __ldcg(reinterpret_cast<const float4*>(p + HI));
         }
-        store8(D.C + (int64_t)row * D.ldc + col, sum, pol);
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            sum[0] = add2(sum[0], pack2(x[u].x, x[u].y));
+            sum[1] = add2(sum[1], pack2(x[u].z, x[u].w));
+            sum[2] = add2(sum[2], pack2(y[u].x, y[u].y));
+            sum[3] = add2(sum[3], pack2(y[u].z, y[u].w));
+        }
     }
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const u64 own = sum[q];
+#pragma unroll
+        for (int j = 1; j < EPS; ++j) sum[q] = add2(sum[q], __shfl_sync(0xffffffffu, own, (lane + j * G) & 31));
+    }
+    if (lane < G) store8<HI>(D.C + (int64_t)row * D.ldc + col, act, act1, sum, pol);
     if (lane == 0) atomicExch(cnt, 0);  // ready for the next launch
 }
 
@@ -208,9 +238,12 @@ template <int G, int FORM>
 struct ContigShape {
     static constexpr int EPS = 32 / G;                       // streams per warp
     // gathers in flight per stream (8 at 4 or 5 CTAs per SM: 0.85-0.89 ms on the power-law graph)
-    static constexpr int DEPTH = 4;
-    static constexpr int BE = G < 16 ? 16 : G;               // entries per batch of a stream
+    static constexpr int DEPTH = G == 4 ? 2 : 4;             // (4 lanes: see contig_ctas)
+    static constexpr int BE = G == 4 ? 8 : G < 16 ? 16 : G;  // entries per batch of a stream
     static constexpr int NB = BE / G;                        // entries a lane loads per batch
+    // a lane's columns: two times 4, HI apart, CW from lane to lane (8 in a row, or, so that lanes of 16-byte
+    // loads read whole lines, 4 in each half of the row)
+    static constexpr int CW = FORM == kFormF32Any ? 4 : 8, HI = FORM == kFormF32Any ? 4 * G : 4;
     static_assert(BE % DEPTH == 0 && DEPTH <= BE, "batches start on a group of DEPTH steps, entries reach DEPTH ahead");
 };
 
@@ -264,7 +297,7 @@ __device__ __forceinline__ void contig_chunk(const ExecDesc* Dp, int32_t c, int 
     // ------------------------------- the chunk and its shares -------------------------------
     unsigned char const* Bl;
     std::conditional_t<form_any(FORM), uint64_t, uint32_t> ldb_bytes;
-    bool act;            // this lane's 8 columns exist
+    bool act, act1;      // this lane's first and second 4 columns exist
     int S, Smin;         // every share has Smin or S nonzeros
     int cnt;             // this share's nonzeros
     int k, k1;           // the next row to store and the first one this share does not store, less k0
@@ -299,9 +332,9 @@ __device__ __forceinline__ void contig_chunk(const ExecDesc* Dp, int32_t c, int 
         }
     };
     // the column id of an entry (bit 31: hot row) gathered into slot u, when `on`
-    auto gather = [&](int32_t e, int u, bool on) {
+    auto gather = [&](int32_t e, int u, bool on, bool on1) {
         const uint32_t col = HOT ? ((uint32_t)e & 0x7fffffffu) : (uint32_t)e;
-        gather8<FORM>(b[u], Bl + (size_t)col * ldb_bytes, HOT && e >= 0 ? pol.first : pol.last, on);
+        gather8<FORM, G>(b[u], Bl + (size_t)col * ldb_bytes, HOT && e >= 0 ? pol.first : pol.last, on, on1);
     };
     {
         const ExecDesc& D = *Dp;
@@ -315,8 +348,9 @@ __device__ __forceinline__ void contig_chunk(const ExecDesc* Dp, int32_t c, int 
             return;                                              // (the same for every warp of a CTA)
         }
         const int sw = ((D.K + nsl - 1) / nsl + 7) & ~7;
-        const int col0 = slice * sw + 8 * li;
-        act = 8 * li < sw && col0 < D.K;
+        const int col0 = slice * sw + Sh::CW * li;
+        act = Sh::CW * li < sw && col0 < D.K;
+        act1 = FORM == kFormF32Any ? Sh::CW * li + Sh::HI < sw && col0 + Sh::HI < D.K : act;
         Bl = reinterpret_cast<const unsigned char*>(D.B) + (int64_t)col0 * ES;
         ldb_bytes = (decltype(ldb_bytes))(D.ldb * ES);
         const int p0 = (total * my) >> lgU, p1 = (total * (my + 1)) >> lgU;
@@ -350,7 +384,7 @@ __device__ __forceinline__ void contig_chunk(const ExecDesc* Dp, int32_t c, int 
 #pragma unroll
         for (int u = 0; u < DEPTH; ++u) {
             b[u] = Gathered<FORM>{};  // inactive lanes hold zeros
-            gather(batg[u * EPS].x, u, act && u < cnt);
+            gather(batg[u * EPS].x, u, act && u < cnt, act1 && u < cnt);
         }
         fetch(2 * BE, cr, vr);  // stored when batch 1 starts
         // the rows of this share: those that end after p0 (from the chunk's start on, for the
@@ -388,7 +422,7 @@ __device__ __forceinline__ void contig_chunk(const ExecDesc* Dp, int32_t c, int 
         park[0] = make_float4(x.x, x.y, y.x, y.y);
         park[1] = make_float4(z.x, z.y, v.x, v.y);
     };
-    auto crow = [&](int q) { return coldp(cold->C) + (int64_t)q * cold64(cold->ldc) + 8 * li; };
+    auto crow = [&](int q) { return coldp(cold->C) + (int64_t)q * cold64(cold->ldc) + Sh::CW * li; };
     // every row that ends at or before entry P, one per share and turn
     auto flush = [&](int P) {
         do {
@@ -396,8 +430,8 @@ __device__ __forceinline__ void contig_chunk(const ExecDesc* Dp, int32_t c, int 
                 if (open) {
                     park_acc();
                     open = false;
-                } else if (act) {
-                    store8(crow(k), acc, pol.first);
+                } else {
+                    store8<Sh::HI>(crow(k), act, act1, acc, pol.first);
                 }
                 acc[0] = acc[1] = acc[2] = acc[3] = 0ull;
                 ++k;
@@ -423,7 +457,7 @@ __device__ __forceinline__ void contig_chunk(const ExecDesc* Dp, int32_t c, int 
         for (int u = 0; u < DEPTH; ++u) {
             if (P + u >= min_end) flush(P + u);
             accumulate<FORM>(acc, __int_as_float(e0[u * EPS].y), b[u]);
-            gather(e1[u * EPS].x, u, act && P + u + DEPTH < cnt);
+            gather(e1[u * EPS].x, u, act && P + u + DEPTH < cnt, act1 && P + u + DEPTH < cnt);
         }
     }
     {
@@ -462,14 +496,14 @@ __device__ __forceinline__ void contig_chunk(const ExecDesc* Dp, int32_t c, int 
     if (tail && !through) {
         const bool ended = chain(acc);
         cut = !ended;
-        if (ended && act) store8(crow(k1), acc, pol.first);
+        if (ended) store8<Sh::HI>(crow(k1), act, act1, acc, pol.first);
     }
     __syncwarp();
     const int32_t k0 = __ldg(&D.chunk_rec[c].k0);
     const int sw = ((D.K + nsl - 1) / nsl + 7) & ~7;
-    const int col0 = slice * sw + 8 * li;
+    const int col0 = slice * sw + Sh::CW * li;
     if (__any_sync(0xffffffffu, cut))
-        deliver_piece(D, k0 + k1, c, cut, act, col0, acc[0], acc[1], acc[2], acc[3], nsl, slice, pol.first);
+        deliver_piece<G, Sh::HI>(D, k0 + k1, c, cut, act, act1, col0, acc[0], acc[1], acc[2], acc[3], nsl, slice, pol.first);
     // the chunk starts inside row k0: its part is the first share's
     const bool head = my == 0 && (__ldg(&D.chunk_rec[c].flags) & kChunkHeadCut);
     if (__any_sync(0xffffffffu, head)) {
@@ -482,15 +516,24 @@ __device__ __forceinline__ void contig_chunk(const ExecDesc* Dp, int32_t c, int 
             if (through) chain(acc);
         }
         __syncwarp();
-        deliver_piece(D, k0, c, head, act, col0, acc[0], acc[1], acc[2], acc[3], nsl, slice, pol.first);
+        deliver_piece<G, Sh::HI>(D, k0, c, head, act, act1, col0, acc[0], acc[1], acc[2], acc[3], nsl, slice, pol.first);
     }
     sync();  // the parked parts and the batch ring are reused by the next chunk
 }
 
-// CTAs per SM: 7 for 16-lane FP32 groups (power-law 0.68 ms; 0.72 ms at 6 and at 5), 5 for the
-// other FP32 widths (512 graphs, K 64: 2.35 ms; 2.39 ms at 7), 6 for BF16 (0.184 ms; 0.203 ms at 5).
-template <int G, int FORM, bool HOT>
-__global__ void __launch_bounds__(kExecThreads, form_bf16(FORM) ? 6 : (G == 16 ? 7 : 5)) k_exec_contig(
+// CTAs per SM, by what is left of the registers for the gather ring (each side measured with the next
+// number up and down):
+//   FP32, 32-byte B, 16 lanes: 5, and 7 where B is past L2 (FAR) and more warps hide HBM's latency, although
+//     7 spill (2^16 / 2^20 nodes of 16, K 128, W 256: 63 / 743 us at 5, 73 / 686 at 7; W 512 58 / 710, 70 / 667)
+//   4 lanes: 6, BF16 7, with a ring of 2 (2^20 nodes, K 32: 338 us; 388 at 5; 446 at 5 with a ring of 4 and
+//     batches of 16)
+//   other FP32 widths 5 (512 graphs, K 64: 2.35 ms; 2.39 at 7), BF16 6 (300007 nodes, K 96: 0.184 ms; 0.203 at 5)
+constexpr int contig_ctas(int G, int form, bool far)
+{
+    return form_bf16(form) ? (G == 4 ? 7 : 6) : G == 4 ? 6 : G == 16 && far ? 7 : 5;
+}
+template <int G, int FORM, bool HOT, bool FAR>
+__global__ void __launch_bounds__(kExecThreads, contig_ctas(G, FORM, FAR)) k_exec_contig(
     const ExecDesc* __restrict__ descs, const int32_t* __restrict__ queue,
     const int32_t* __restrict__ queue_desc, int64_t n_items, int32_t* ctrl, int32_t nsl, int32_t coop,
     const __grid_constant__ ExecDesc d0)
@@ -549,12 +592,16 @@ typedef void (*ContigKernel)(const ExecDesc*, const int32_t*, const int32_t*, in
                              ExecDesc);
 
 template <int FORM, bool HOT>
-static ContigKernel pick_lanes(int width)
+static ContigKernel pick_lanes(int width, bool far = false)
 {
-    if (width <= 32) return k_exec_contig<4, FORM, HOT>;
-    if (width <= 64) return k_exec_contig<8, FORM, HOT>;
-    if (width <= 128) return k_exec_contig<16, FORM, HOT>;
-    return k_exec_contig<32, FORM, HOT>;
+    if (width <= 32) return k_exec_contig<4, FORM, HOT, false>;
+    if (width <= 64) return k_exec_contig<8, FORM, HOT, false>;
+    if (width <= 128) {
+        if constexpr (FORM == kFormF32)
+            if (far) return k_exec_contig<16, FORM, HOT, true>;
+        return k_exec_contig<16, FORM, HOT, false>;
+    }
+    return k_exec_contig<32, FORM, HOT, false>;
 }
 
 static ContigKernel pick_contig(int K, bool bf16, const ContigMode& m)
@@ -564,13 +611,27 @@ static ContigKernel pick_contig(int K, bool bf16, const ContigMode& m)
     if (m.any)  // (the hot map is only a cache hint)
         return bf16 ? pick_lanes<kFormBf16Any, false>(width) : pick_lanes<kFormF32Any, false>(width);
     if (bf16) return m.hot ? pick_lanes<kFormBf16, true>(width) : pick_lanes<kFormBf16, false>(width);
-    return m.hot ? pick_lanes<kFormF32, true>(width) : pick_lanes<kFormF32, false>(width);
+    return m.hot ? pick_lanes<kFormF32, true>(width, m.far) : pick_lanes<kFormF32, false>(width, m.far);
 }
 
 const void* contig_kernel(int K, bool bf16, const ContigMode& m)
 {
     return reinterpret_cast<const void*>(pick_contig(K, bf16, m));
 }
+
+// Past L2 (K 128 FP32, us at 5 and at 7 CTAs an SM: 2^17 nodes, 67 MB, W 256 97 and 109; 2^18 nodes, 134 MB,
+// 180 and 185; 2^19 nodes, 268 MB, 361 and 350; 2^20 nodes 741 and 692).
+bool contig_far(int64_t n, int K, bool bf16, int device)
+{
+    return n * ((K + contig_slices(K) - 1) / contig_slices(K)) * (bf16 ? 2 : 4) > l2_bytes(device);
+}
+
+// At most 8 chunks per SM, while the launch has 20 to 28 warps there: with one chunk a warp most
+// warps would have none, and sharing a chunk among four shortens its chain of steps (4096 rows of
+// 16, 272 chunks: 25.5 -> 13.5 us a call).  For a plan it depends on the plan alone, so that a
+// request sums its rows in the same order whatever shares its launch; a batch decides for all of its graphs
+// of a width together.
+bool contig_coop(int64_t n_chunks, int device) { return n_chunks <= 8 * (int64_t)num_sms(device); }
 
 // the persistent grid: resident CTAs on every SM, at most one per unit of work
 ns_status_t contig_prepare(int64_t n_items, int K, bool bf16, const ContigMode& m, int* grid_out)

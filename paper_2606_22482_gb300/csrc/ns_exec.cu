@@ -105,11 +105,13 @@ bool plan_contig(const Plan* P)
     return P->tune.tau_tile == kTauInf && P->st.n_dwin == 0 && P->st.n_rl == P->st.m;
 }
 
-// At most 8 chunks per SM, while the launch has 20 to 28 warps there: with one chunk a warp most
-// warps would have none, and sharing a chunk among four shortens its chain of steps (4096 rows of
-// 16, 272 chunks: 25.5 -> 13.5 us a call).  A plan's own property (not a launch's), so that a
-// request sums its rows in the same order whatever shares its launch.
-bool plan_coop(const Plan* P) { return P->st.n_chunks <= 8 * (int64_t)num_sms(P->device); }
+// Column slices start every chunk once a slice, which costs more than they gain when a chunk is a few
+// nonzeros (K 512 FP32, 2^16 nodes of 16, us by slices and by k_exec: W 128 197 and 225, 64 261 and 241, 32 385
+// and 290, 16 653 and 389).
+bool contig_form(const Plan* P, int K)
+{
+    return plan_contig(P) && !(contig_slices(K) > 1 && P->tune.chunk_nnz <= 32);
+}
 
 void fill_desc(const Plan* P, const void* B, int64_t ldb, float* C, int64_t ldc, ExecDesc* d)
 {
@@ -199,6 +201,18 @@ int num_sms(int device)
     return cached[device];
 }
 
+int64_t l2_bytes(int device)
+{
+    static int64_t cached[64] = {0};
+    if (device < 0 || device >= 64) return 126ll << 20;
+    if (!cached[device]) {
+        int v = 0;
+        if (cudaDeviceGetAttribute(&v, cudaDevAttrL2CacheSize, device) != cudaSuccess || v <= 0) v = 126 << 20;
+        cached[device] = v;
+    }
+    return cached[device];
+}
+
 // dynamic shared memory of one execute CTA: the dense item's tiles (phase 1) or the residual
 // warps' staging rings (phase 2), whichever is larger
 static size_t exec_smem_bytes(int K, int TM, int TK, bool bf16, bool dense, int W)
@@ -280,7 +294,7 @@ ns_status_t exec_launch(const ExecDesc* descs, const int32_t* queue, const int32
 ns_status_t exec_launch_plan(Plan* P, cudaStream_t s)
 {
     const int K = P->desc_host.K;  // the column slice of this launch
-    const bool contig = plan_contig(P);
+    const bool contig = contig_form(P, K);
     const bool any = contig && contig_any(P->desc_host.B, P->desc_host.ldb, P->dtype == NS_BF16);
     int* gc = K == P->K ? &P->exec_grid[any] : &P->exec_grid_slice[any];
     if (K != P->K && P->exec_grid_slice_K[any] != K) {
@@ -291,8 +305,8 @@ ns_status_t exec_launch_plan(Plan* P, cudaStream_t s)
         ContigMode m;
         m.any = any;
         m.hot = P->hot_bits != nullptr;
-        m.coop = plan_coop(P);
-        m.W = P->tune.chunk_nnz;
+        m.far = contig_far(P->st.n, K, P->dtype == NS_BF16, P->device);
+        m.coop = contig_coop(P->st.n_chunks, P->device);
         return contig_launch(nullptr, P->queue, nullptr, P->st.n_items, P->ctrl, K, P->dtype == NS_BF16, m, gc, s,
                              &P->desc_host);
     }

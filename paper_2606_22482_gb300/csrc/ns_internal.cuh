@@ -231,13 +231,14 @@ ns_status_t window_pass(Plan* P, WindowResult* W, cudaStream_t s);
 __host__ __device__ inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 int num_sms(int device);
+int64_t l2_bytes(int device);
 
 // form of a contiguous-stream launch (ns_contig.cu)
 struct ContigMode {
     bool any = false;   // FP32 rows of B off the 32-byte boundaries, or rows 4 GB or more apart (contig_any)
+    bool far = false;   // the launch's B together are past L2 (contig_far)
     bool hot = false;   // single plan with a hot-row map (l2_hints = 2)
-    bool coop = false;  // the warps of a CTA share a chunk (plan_coop)
-    int W = 256;        // chunk_nnz of the launch's plans
+    bool coop = false;  // the warps of a CTA share a chunk (contig_coop)
 };
 // Column slices of a contiguous-stream launch: one pass up to K = 256, then 128 columns a slice,
 // so that a slice's rows of B stay in L2 and no lane group is wider than a warp.
@@ -267,7 +268,7 @@ ns_status_t f32_launch(const ExecDesc* descs, const int32_t* queue, const int32_
                        int32_t* ctrl, int K, int TM, int TK, bool hint, int W, int* grid_cache, cudaStream_t s,
                        const ExecDesc* d0);
 bool plan_contig(const Plan* P);  // contiguous residual stream (tau_tile = inf)
-bool plan_coop(const Plan* P);    // ... with so few chunks that the warps of a CTA share one
+bool contig_form(const Plan* P, int K);  // ... and launches of K columns take k_exec_contig
 ns_status_t contig_launch(const ExecDesc* descs, const int32_t* queue, const int32_t* queue_desc, int64_t n_items,
                           int32_t* ctrl, int K, bool bf16, const ContigMode& m, int* grid_cache, cudaStream_t s,
                           const ExecDesc* d0 = nullptr);
@@ -276,6 +277,10 @@ inline bool contig_any(const void* B, int64_t ldb, bool bf16)
 {
     return ldb > (int64_t)UINT32_MAX / (bf16 ? 2 : 4) || (!bf16 && (reinterpret_cast<uintptr_t>(B) & 31u) != 0);
 }
+// the columns of one pass over n rows of B are past L2
+bool contig_far(int64_t n, int K, bool bf16, int device);
+// so few chunks that the warps of a CTA share one
+bool contig_coop(int64_t n_chunks, int device);
 ns_status_t contig_prepare(int64_t n_items, int K, bool bf16, const ContigMode& m, int* grid_out);
 const void* contig_kernel(int K, bool bf16, const ContigMode& m);  // (all of them take the same arguments)
 ns_status_t plan_create(const ns_csr_t* A, int32_t K, ns_dtype_t dt, const ns_tune_t* tune,

@@ -589,10 +589,12 @@ static void launch_group(Server* S, std::vector<SReq*>& rs, int cls, int K, bool
     cudaEventRecord(L.up_ev, es);
     cudaStreamWaitEvent(es, L.h2d_ev, 0);
     // every plan of a group has the same form (part of the group's key); B starts on a 256-byte block
-    const bool contig = plan_contig(rs[0]->sp->plan);
+    const bool contig = contig_form(rs[0]->sp->plan, K);
     ContigMode mode;
-    mode.coop = plan_coop(rs[0]->sp->plan);
-    mode.W = S->cfg.tune.chunk_nnz;
+    int64_t n_rows = 0;
+    for (const SReq* q : rs) n_rows += S->graphs[q->r.graph_id].n;
+    mode.far = contig_far(n_rows, K, bf16, S->device);
+    mode.coop = contig_coop(rs[0]->sp->plan->st.n_chunks, S->device);
     // a bulk launch leaves a quarter of the GPU free, so small requests' launches start at once
     int grid = 0;
     if (cls) {
@@ -727,7 +729,7 @@ static void worker_loop(Server* S)
                 const Plan* P = q->sp->plan;
                 // kernel form: plans with few chunks take the cooperative form, so they launch apart, and
                 // so do FP32 plans that keep their dense tiles' planes
-                const int form = plan_contig(P) ? (plan_coop(P) ? 2 : 1) : plan_planes(P) ? 3 : 0;
+                const int form = contig_form(P, q->r.K) ? (contig_coop(P->st.n_chunks, S->device) ? 2 : 1) : plan_planes(P) ? 3 : 0;
                 groups[{q->cls, q->r.K, (int)q->r.b_dtype, P->st.n_dwin > 0 ? 1 : 0, P->tune.TM, P->tune.TK, form}]
                     .push_back(q);
             }
