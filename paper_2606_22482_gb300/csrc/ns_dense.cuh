@@ -12,6 +12,8 @@
 //              x = hi + lo with hi = tf32(x), lo = tf32(x - hi); a*b ~ ahi*bhi + ahi*blo + alo*bhi,
 //              which keeps the error near FP32 while running on the tensor pipe.
 //
+// It serves K > 256, and FP32 plans of any K whose tiles keep no planes (ns_exec_f32.cu has the others).
+//
 // The window's TM x K result is assembled in shared memory, the rows' absorbed residual is
 // added on the CUDA cores and each row is delivered (stored, or written as piece 0 of a split
 // row).  The CTA's four warps split the window as TM/16 row groups x 4/(TM/16) column groups.

@@ -1,9 +1,9 @@
-// ns_exec_f32.cu -- the persistent kernel of FP32 plans with dense tiles (K <= 256): the dense item
-// on the 5th-generation tensor cores.
+// ns_exec_f32.cu -- the persistent kernel of FP32 plans that keep their dense tiles' planes (K <= 256): the
+// dense item on the 5th-generation tensor cores.
 //
 // FP32 operands run as three BF16 pieces each, x = x0 + x1 + x2 (x0 by truncation, so that it never
-// overflows; x1 and x2 rounded to nearest; 24 bits in all), and the product keeps the six terms
-// above 2^-24: a0 b0 | a0 b1 + a1 b0 | a1 b1 + a0 b2 + a2 b0, in three accumulators X0 | X1 | X2 by
+// overflows; x1 and x2 rounded to nearest; 24 bits in all), and the product keeps the six largest
+// terms (what is left out is below 2^-22 of |a b|: a truncated x0 leaves x1 up to 2^-7 of x): a0 b0 | a0 b1 + a1 b0 | a1 b1 + a0 b2 + a2 b0, in three accumulators X0 | X1 | X2 by
 // size.  The tensor pipe's FP32 accumulation is not round-to-nearest, so a tile's a0 b0 starts a
 // fresh X0 (two alternate), which is added to the window's sum in registers with an ordinary FP32
 // add; X1 and X2, 2^-8 and 2^-16 of the result, accumulate over the window.
@@ -27,6 +27,9 @@
 // on 152 SMs are 3.4 rounds of about 33 us; a tile takes about 0.8 us, its eight small MMAs and the
 // producers' splits about half of that each way, and a window's delivery adds 4 us.  Traffic (240 MB
 // of planes from HBM) and the tensor pipe (31 GFLOP of pieces) would each allow about 35 us.
+// Other widths and tiles, against the mma.sync item (us an execute): mask 8192, TM 16, TK 16, K 8 127 -> 86,
+// K 32 126 -> 86, K 256 258 -> 149; TM 64, TK 32, K 8 102 -> 29, K 64 160 -> 29; RMAT 2^15, TM 16, TK 16, tau 32,
+// K 8 to 32, where the residual decides, 148 on both sides: nowhere slower, so K alone is the rule.
 // Also tried: all operands of an MMA computed by the issuing lane alone (100 cycles an MMA), loads of
 // one feature a lane (32 instructions a tile and warp, 90 cycles each): 213 to 276 us.
 //
@@ -283,43 +286,43 @@ __device__ bool ts_window_product(const ExecDesc& D, int32_t w, unsigned char* s
         const uint32_t lanes = (uint32_t)(32 * warp) << 16;
         const int32_t Kw = D.K;
         for (int j = 1; j <= J; ++j) {
-                            const uint32_t g = g0 + (uint32_t)(j - 1), s = g & 1u;
-                            if (ok && !mbar_wait(bars + kTsAccFull + s, (g >> 1) & 1u)) ok = false;
-                            __syncwarp();
-                            tc_fence_after();
-            #pragma unroll
-                            for (int c0 = 0; c0 < 64; c0 += 16) {
-                                if (c0 < TM) {
-                                    uint32_t r[16];
-                                    tc_ld16(S.tmem + lanes + s * (uint32_t)TM + c0, r);
-            #pragma unroll
-                                    for (int q = 0; q < 16; ++q) acc[c0 + q] += __uint_as_float(r[q]);
-                                }
-                            }
-                            if (j == T || j == J) {  // a feature block is complete (with it X1 and X2)
-            #pragma unroll
-                                for (int c0 = 0; c0 < 64; c0 += 16) {
-                                    if (c0 < TM) {
-                                        uint32_t r[16], q2[16];
-                                        tc_ld16(S.tmem + lanes + kTsX1 + TM + c0, q2);
-                                        tc_ld16(S.tmem + lanes + kTsX1 + c0, r);
-            #pragma unroll
-                                        for (int q = 0; q < 16; ++q)
-                                            acc[c0 + q] += __uint_as_float(r[q]) + __uint_as_float(q2[q]);
-                                    }
-                                }
-                            }
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(bars + kTsAccEmpty + s);
-                            if (j == T || j == J) {
-                                const int f = (j == T ? 0 : 128) + 32 * warp + lane;
-            #pragma unroll
-                                for (int q = 0; q < 64; ++q) {
-                                    if (q < TM && f < Kw) Cs[q * G.cs_stride + f] = acc[q];
-                                    acc[q] = 0.f;
-                                }
-                            }
+            const uint32_t g = g0 + (uint32_t)(j - 1), s = g & 1u;
+            if (ok && !mbar_wait(bars + kTsAccFull + s, (g >> 1) & 1u)) ok = false;
+            __syncwarp();
+            tc_fence_after();
+#pragma unroll
+            for (int c0 = 0; c0 < 64; c0 += 16) {
+                if (c0 < TM) {
+                    uint32_t r[16];
+                    tc_ld16(S.tmem + lanes + s * (uint32_t)TM + c0, r);
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) acc[c0 + q] += __uint_as_float(r[q]);
+                }
+            }
+            if (j == T || j == J) {  // a feature block is complete (with it X1 and X2)
+#pragma unroll
+                for (int c0 = 0; c0 < 64; c0 += 16) {
+                    if (c0 < TM) {
+                        uint32_t r[16], q2[16];
+                        tc_ld16(S.tmem + lanes + kTsX1 + TM + c0, q2);
+                        tc_ld16(S.tmem + lanes + kTsX1 + c0, r);
+#pragma unroll
+                        for (int q = 0; q < 16; ++q)
+                            acc[c0 + q] += __uint_as_float(r[q]) + __uint_as_float(q2[q]);
+                    }
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bars + kTsAccEmpty + s);
+            if (j == T || j == J) {
+                const int f = (j == T ? 0 : 128) + 32 * warp + lane;
+#pragma unroll
+                for (int q = 0; q < 64; ++q) {
+                    if (q < TM && f < Kw) Cs[q * G.cs_stride + f] = acc[q];
+                    acc[q] = 0.f;
+                }
+            }
         }
     }
     S.g = g0 + (uint32_t)J;
@@ -435,8 +438,8 @@ static F32Kernel pick_f32(int K, bool hint)
     return hint ? k_exec_f32<2, true> : k_exec_f32<2, false>;
 }
 
-// Dynamic shared memory, and the warps of a CTA that take residual chunks: all twelve while their
-// staging areas fit, never fewer than the four that always do.
+// Dynamic shared memory, and the warps of a CTA that take residual chunks: all of them
+// while their staging areas fit, never fewer than the four that always do.
 static size_t f32_smem(int K, int TM, int TK, int W, int* res_warps)
 {
     const int wb = stage_geom(K, false, W).warp_bytes;

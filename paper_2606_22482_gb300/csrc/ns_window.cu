@@ -731,7 +731,7 @@ __global__ void __launch_bounds__(kWinThreads, 4) k_emit_tiles(EmitArgs a)
     for (int r = warp; r < nrows; r += nwarps) {
         const int64_t rend = rb0[r + 1];
         for (int64_t eb = rb0[r]; eb < rend; eb += 128) {  // four positions per lane in flight
-            int32_t pv[4], iv[4];
+            int32_t pv[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int64_t e = eb + 32 * u + lane;
