@@ -6,8 +6,8 @@
 //
 // What bounds it: every nonzero gathers one B row (4 K or 2 K bytes) from L2 into an SM.  A kernel
 // that only gathers the same column streams moves 21 TB/s (power-law graph of 2^20 nodes, 512-byte
-// rows, 0.39 ms).  This one moves 12.6 TB/s there: the rest of the time goes to instructions around
-// the gathers (54 per step of two nonzeros; row ends take most of what is not the product itself)
+// rows, 0.39 ms).  This one moves 12.8 TB/s there: the rest of the time goes to instructions around
+// the gathers (53 per step of two nonzeros; row ends take most of what is not the product itself)
 // and to the starts of chunks (about 10 us each, a chain of dependent loads).
 //
 // Split of the work: a lane owns 8 adjacent columns (32 bytes of FP32 in one 256-bit load, or 16
@@ -148,12 +148,12 @@ __device__ __forceinline__ void store8(float* p, bool act, bool act1, const u64 
 // a group of G lanes stands for: 4 from `col` where `act` and 4 from col + HI where `act1`.  The piece that
 // arrives last sums the pieces and stores the row: lane group j adds pieces j, j + 32 / G, ... in order,
 // kAhead of them on their way at a time, then the groups' sums are added in order.
-template <int G, int HI>
+template <int G, int HI, int kAhead>
 __device__ __noinline__ void deliver_piece(const ExecDesc& D, int32_t row, int32_t c, bool mine, bool act, bool act1,
                                            int col, u64 a0, u64 a1, u64 a2, u64 a3, int nsl, int slice,
                                            uint64_t pol)
 {
-    constexpr int EPS = 32 / G, kAhead = G < 32 ? 2 : 4;
+    constexpr int EPS = 32 / G;
     const int lane = threadIdx.x & 31;
     const unsigned who = __ballot_sync(0xffffffffu, mine);
     if (who == 0u) return;
@@ -271,7 +271,7 @@ __device__ __forceinline__ int64_t cold64(const int64_t& x) { return *const_cast
 
 // HOT: the planner's hot-row map picks each gather's L2 policy; its bit travels as bit 31 of the
 // column id.
-template <int G, int FORM, bool HOT>
+template <int G, int FORM, bool HOT, bool FAR>
 __device__ __forceinline__ void contig_chunk(const ExecDesc* Dp, int32_t c, int slice, int nsl, int lgU, int lane,
                                              int warp, const ContigPolicies& pol, float4* park0, int2* bat,
                                              int32_t* through0, ContigCold* cold)
@@ -281,6 +281,9 @@ __device__ __forceinline__ void contig_chunk(const ExecDesc* Dp, int32_t c, int 
     constexpr int ES = form_bf16(FORM) ? 2 : 4;
     constexpr int lgE = EPS == 1 ? 0 : EPS == 2 ? 1 : EPS == 4 ? 2 : 3;
     const int g = lane / G, li = lane % G;
+    // pieces of a split row on their way at a time (what the call saves counts in this kernel's registers:
+    // power-law 2^20, K 128, 676 us with 4, 675 with 2, 670 with 1; 2^20 nodes, K 64 467 with 4, 456 with 2)
+    constexpr int AHEAD = FAR ? 1 : G < 32 ? 2 : 4;
     const bool coop = lgU != lgE;  // the CTA's four warps share the chunk
     const int U = 1 << lgU;        // shares (streams) of the chunk
     const int u0 = warp * EPS;     // this warp's first share (warp is 0 in the one-warp form)
@@ -503,7 +506,7 @@ __device__ __forceinline__ void contig_chunk(const ExecDesc* Dp, int32_t c, int 
     const int sw = ((D.K + nsl - 1) / nsl + 7) & ~7;
     const int col0 = slice * sw + Sh::CW * li;
     if (__any_sync(0xffffffffu, cut))
-        deliver_piece<G, Sh::HI>(D, k0 + k1, c, cut, act, act1, col0, acc[0], acc[1], acc[2], acc[3], nsl, slice, pol.first);
+        deliver_piece<G, Sh::HI, AHEAD>(D, k0 + k1, c, cut, act, act1, col0, acc[0], acc[1], acc[2], acc[3], nsl, slice, pol.first);
     // the chunk starts inside row k0: its part is the first share's
     const bool head = my == 0 && (__ldg(&D.chunk_rec[c].flags) & kChunkHeadCut);
     if (__any_sync(0xffffffffu, head)) {
@@ -516,7 +519,7 @@ __device__ __forceinline__ void contig_chunk(const ExecDesc* Dp, int32_t c, int 
             if (through) chain(acc);
         }
         __syncwarp();
-        deliver_piece<G, Sh::HI>(D, k0, c, head, act, act1, col0, acc[0], acc[1], acc[2], acc[3], nsl, slice, pol.first);
+        deliver_piece<G, Sh::HI, AHEAD>(D, k0, c, head, act, act1, col0, acc[0], acc[1], acc[2], acc[3], nsl, slice, pol.first);
     }
     sync();  // the parked parts and the batch ring are reused by the next chunk
 }
@@ -569,7 +572,7 @@ __global__ void __launch_bounds__(kExecThreads, contig_ctas(G, FORM, FAR)) k_exe
         if (!D.rl_all) {  // guard: launched for a plan without a contiguous residual stream
             if (lane == 0) atomicOr(D.status, kStatusInternal);
         } else if (c >= 0 && c < D.n_chunks) {
-            contig_chunk<G, FORM, HOT>(&D, (int32_t)c, slice, nsl, coop ? lgE + 2 : lgE, lane, coop ? warp : 0, pol,
+            contig_chunk<G, FORM, HOT, FAR>(&D, (int32_t)c, slice, nsl, coop ? lgE + 2 : lgE, lane, coop ? warp : 0, pol,
                                        park0, s_bat[warp], through0, s_cold + warp);
         }
         if (coop) {
