@@ -140,10 +140,9 @@ EXEC_SOURCES = ("ns_exec.cu", "ns_contig.cu", "ns_exec_f32.cu", "ns_residual.cuh
                 "ns_internal.cuh", "ns_dense.cuh", "ns_dense_tc.cuh", "ns_ptx.cuh")
 MEASURED_TRAFFIC = {
     # (workload, tau_tile, chunk_nnz, l2_hints): (source digest, bytes per launch)
-    ("powerlaw", 2147483647, 512, 1): ("ce2d73446f053432", 1676767488 + 542345216),
-    ("powerlaw", 2147483647, 256, 1): ("ce2d73446f053432", 1699133952 + 585530112),
-    ("powerlaw", 2147483647, 512, 2): ("ce2d73446f053432", 1520246272 + 536258048),
-    ("powerlaw", 2147483647, 1024, 1): ("ce2d73446f053432", 1670158080 + 531273984),
+    ("powerlaw", 2147483647, 512, 1): ("c218fd6215f19630", 1772762112 + 551939072),
+    ("powerlaw", 2147483647, 256, 1): ("c218fd6215f19630", 1786630656 + 597434624),
+    ("powerlaw", 2147483647, 1024, 1): ("c218fd6215f19630", 1757437440 + 535467776),
 }
 
 
